@@ -112,7 +112,7 @@ __device__ __forceinline__ CountSum batch_consume_body(const unsigned char* slot
                                                        const ConsCol& c, int lane)
 {
     uint64_t cnt = 0, sum = 0;
-    const Lanes L = make_lanes<B>(c.lo, c.wm1);
+    const Keys<B, BRANCHY> L = make_keys<B, BRANCHY>(c.lo, c.wm1);
     const uint32_t nfull = m.tail ? m.nk - 1u : m.nk;
     scan_tile<B, BRANCHY>(slot, nfull, lane, L, c.lo, c.wm1, cnt, sum);
     if (m.tail) {

@@ -636,8 +636,7 @@ scan_status enqueue_scan(scan_column* c, scan_pred pred, scan_strategy strategy,
         const bool branchy = op == gb::kOpFullBR;
         if (op != gb::kOpFullBF && op != gb::kOpFullBR)
             return fail(SCAN_EINVAL, "zone-skip strategies need a lane-interleaved column");
-        if (c->layout == SCAN_LAYOUT_ROWMAJOR) op = branchy ? gb::kOpRowBR : gb::kOpRowBF;
-        else op = branchy ? gb::kOpBytesBR : gb::kOpBytesBF;
+        op = branchy ? gb::kOpRowBR : gb::kOpRowBF;  // a byte array is the row-major stream's bytes
     } else if (c->layout != SCAN_LAYOUT_LANES && op != gb::kOpFullBF && op != gb::kOpFullBR) {
         return fail(SCAN_EINVAL, "zone-skip strategies need a lane-interleaved column");
     }
@@ -1068,7 +1067,8 @@ scan_status scan_launch_shape(uint32_t b, uint32_t* sms, uint32_t* ctas, uint32_
 {
     g_err.clear();
     if (b < 1 || b > 32) return fail(SCAN_EINVAL, "b must be in 1..32");
-    const gb::LaunchShape si = gb_shape_for(static_cast<int>(b), gb::kOpFullBF);
+    gb::LaunchShape si = gb_shape_for(static_cast<int>(b), gb::kOpFullBF);
+    if (gb::sliced(static_cast<int>(b), false)) si = gb::filled(static_cast<int>(b), si);
     if (sms) *sms = static_cast<uint32_t>(device_info().sms);
     if (ctas) *ctas = static_cast<uint32_t>(persistent_grid());
     if (warps_per_cta) *warps_per_cta = static_cast<uint32_t>(si.warps);

@@ -42,33 +42,46 @@ cudaError_t launch_one(const ScanParams& p, const LaunchShape& sh, int grid, cud
     return cudaGetLastError();
 }
 
-// Full scans: the 16-warp-bound instantiation for CTAs above 8 warps; the
-// branchy vote group per row where the shape asks for it (b <= 21).
+// Full scans.  Bit-sliced widths take one lane per thread and one vote per two
+// blocks: every vote form and geometry of their shape runs the same kernel.  The
+// others: the 16-warp-bound instantiation for CTAs above 8 warps, the 2-lane
+// geometry and the branchy vote form the shape asks for.
 template <int B, bool BRANCHY>
 cudaError_t launch_full(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
 {
-    if constexpr (B >= 9 && B <= 16) {  // the 2-lane geometry: 16-warp bound only
-        if (sh.vec_lanes == 2) {
-            if constexpr (BRANCHY) {
-                if (sh.vote_rows == 3) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 3, 2>>(p, sh, grid, st);
-                if (sh.vote_rows == 2) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 2, 2>>(p, sh, grid, st);
-                if (sh.vote_rows) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 1, 2>>(p, sh, grid, st);
-            }
-            return launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16, 0, 2>>(p, sh, grid, st);
+    if constexpr (sliced(B, BRANCHY)) {
+        return launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16>>(p, filled(B, sh), grid, st);
+    } else {
+        if constexpr (!BRANCHY && B <= 16) {  // the 2-lane geometry: 16-warp bound only
+            if (sh.vec_lanes == 2) return launch_one<B, k_scan_full<B, false, kLayLanes, 16, 0, 2>>(p, sh, grid, st);
         }
+        if (sh.vec_lanes != 0 && sh.vec_lanes != default_lpt(B)) return cudaErrorInvalidValue;
+        const bool w16 = sh.warps > 8;
+        if constexpr (BRANCHY && B <= 21) {
+            // the PTX row vote: the 16-warp bound only (any CTA up to 16 warps)
+            if (sh.vote_rows == 3) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 3>>(p, sh, grid, st);
+            if (sh.vote_rows == 2) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 2>>(p, sh, grid, st);
+            if (sh.vote_rows)
+                return w16 ? launch_one<B, k_scan_full<B, true, kLayLanes, 16, 1>>(p, sh, grid, st)
+                           : launch_one<B, k_scan_full<B, true, kLayLanes, 8, 1>>(p, sh, grid, st);
+        }
+        if constexpr (BRANCHY && branchy_filled(B)) {
+            const LaunchShape f = filled(B, sh);
+            if (f.warps > 8) return launch_one<B, k_scan_full<B, true, kLayLanes, 16>>(p, f, grid, st);
+        }
+        return w16 ? launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16>>(p, sh, grid, st)
+                   : launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 8>>(p, sh, grid, st);
     }
-    if (sh.vec_lanes != 0 && sh.vec_lanes != default_lpt(B)) return cudaErrorInvalidValue;
-    const bool w16 = sh.warps > 8;
-    if constexpr (BRANCHY && B <= 21) {
-        // the PTX row vote: the 16-warp bound only (any CTA up to 16 warps)
-        if (sh.vote_rows == 3) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 3>>(p, sh, grid, st);
-        if (sh.vote_rows == 2) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 2>>(p, sh, grid, st);
-        if (sh.vote_rows)
-            return w16 ? launch_one<B, k_scan_full<B, true, kLayLanes, 16, 1>>(p, sh, grid, st)
-                       : launch_one<B, k_scan_full<B, true, kLayLanes, 8, 1>>(p, sh, grid, st);
-    }
-    return w16 ? launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16, 0>>(p, sh, grid, st)
-               : launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 8, 0>>(p, sh, grid, st);
+}
+
+// Full scans of row-major columns.
+template <int B, bool BRANCHY>
+cudaError_t launch_row(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
+{
+    if constexpr (sliced(B, BRANCHY, row_decode(B)) || BRANCHY)
+        return launch_one<B, k_scan_full<B, BRANCHY, kLayRow, 16>>(p, filled(B, sh), grid, st);
+    else
+        return launch_one<B, k_scan_full<B, BRANCHY, kLayRow>>(p, sh, grid, st);
 }
 
 template <int B>
@@ -81,15 +94,8 @@ cudaError_t launch_b(int op, const ScanParams& p, const LaunchShape& sh, int gri
     case kOpQueueBF: return launch_one<B, k_scan_queue<B, false>>(p, sh, grid, st);
     case kOpQueueBR: return launch_one<B, k_scan_queue<B, true>>(p, sh, grid, st);
     case kOpZoneBuild: return launch_one<B, k_zonemap_build<B>>(p, sh, grid, st);
-    case kOpRowBF: return launch_one<B, k_scan_full<B, false, kLayRow>>(p, sh, grid, st);
-    case kOpRowBR: return launch_one<B, k_scan_full<B, true, kLayRow>>(p, sh, grid, st);
-    case kOpBytesBF:
-    case kOpBytesBR:
-        if constexpr (B == 8 || B == 16) {
-            if (op == kOpBytesBF) return launch_one<B, k_scan_full<B, false, kLayBytes>>(p, sh, grid, st);
-            return launch_one<B, k_scan_full<B, true, kLayBytes>>(p, sh, grid, st);
-        }
-        return cudaErrorInvalidValue;
+    case kOpRowBF: return launch_row<B, false>(p, sh, grid, st);
+    case kOpRowBR: return launch_row<B, true>(p, sh, grid, st);
     default: return cudaErrorInvalidValue;
     }
 }

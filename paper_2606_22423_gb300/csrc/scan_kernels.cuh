@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "gb_ptx.cuh"
+#include "slice.cuh"
 
 namespace gb {
 
@@ -63,10 +64,11 @@ __host__ __device__ constexpr int default_lpt(int b) { return b <= 16 ? 4 : 2; }
 
 template <int B, int LPT = default_lpt(B)>
 struct Geo {
-    static_assert(LPT == 2 || LPT == 4, "2 or 4 lanes per thread");
+    static_assert(LPT == 1 || LPT == 2 || LPT == 4, "1, 2 or 4 lanes per thread");
     static constexpr int kLpt = LPT;
     static constexpr int kTpb = 32 / kLpt;
-    using Vec = typename std::conditional<kLpt == 4, uint4, uint2>::type;
+    using Vec = typename std::conditional<kLpt == 4, uint4,
+                                          typename std::conditional<kLpt == 2, uint2, uint32_t>::type>::type;
 };
 
 // Default launch shape for width B (used until a tuned shape is installed):
@@ -134,6 +136,7 @@ __device__ __forceinline__ uint32_t lane_word(const uint4& v, int k)
     return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
 }
 __device__ __forceinline__ uint32_t lane_word(const uint2& v, int k) { return k == 0 ? v.x : v.y; }
+__device__ __forceinline__ uint32_t lane_word(uint32_t v, int) { return v; }
 
 // Code of row r for the thread's lane k (r, k compile-time after unrolling).
 template <int B, int LPT = default_lpt(B)>
@@ -158,6 +161,23 @@ __device__ __forceinline__ void load_rows(typename Geo<B, LPT>::Vec (&W)[B], con
 {
 #pragma unroll
     for (int w = 0; w < B; ++w) W[w] = rows[w * Geo<B, LPT>::kTpb];
+}
+
+// The 32 codes of a block that this lane decodes, as B words in stream order.
+// Lane layout: the lane's own stream, word w at 32w + lane.  Row-major: segment s of the thread is the block's
+// segment lane + 32s of m whole words, D whole codes; m is odd, so the lanes'
+// reads at a stride of m words fall in distinct banks.
+template <int B, int LAY>
+__device__ __forceinline__ void load_stream(uint32_t (&W)[B], const uint32_t* words, int lane)
+{
+    if constexpr (LAY == kLayLanes) {
+#pragma unroll
+        for (int w = 0; w < B; ++w) W[w] = words[32 * w + lane];
+    } else {
+        constexpr int kM = slice_odd(B);
+#pragma unroll
+        for (int w = 0; w < B; ++w) W[w] = words[(lane + 32 * (w / kM)) * kM + w % kM];
+    }
 }
 
 // -------------------------------------------------------------- aggregate
@@ -207,6 +227,18 @@ __device__ __forceinline__ Lanes make_lanes(uint32_t lo, uint32_t wm1)
     L.negloi = 0u - L.loi;
     L.wm1 = wm1;
     return L;
+}
+
+// What a kernel keeps of the predicate: slice keys for the bit-sliced widths,
+// the packed-add constants above for the others.
+template <int B, bool BRANCHY, int LAY = kLayLanes>
+using Keys = typename std::conditional<sliced(B, BRANCHY, LAY), SliceKeys<B>, Lanes>::type;
+
+template <int B, bool BRANCHY, int LAY = kLayLanes>
+__device__ __forceinline__ Keys<B, BRANCHY, LAY> make_keys(uint32_t lo, uint32_t wm1)
+{
+    if constexpr (sliced(B, BRANCHY, LAY)) return make_slice_keys<B>(lo, wm1, opaque_one());
+    else return make_lanes<B>(lo, wm1);
 }
 
 // True when row r's field sits at the top of its word (extracted by IMAD.HI).
@@ -360,41 +392,6 @@ template <bool TOP, int LPT>
 __device__ __forceinline__ void branchy_row(uint32_t (&a)[LPT], const uint32_t (&u)[LPT], const Lanes& L);
 
 template <>
-__device__ __forceinline__ void branchy_row<true, 4>(uint32_t (&a)[4], const uint32_t (&u)[4], const Lanes& L)
-{
-    asm volatile(
-        "{\n\t.reg .pred p0, p1, p2, p3, q;\n\t.reg .b32 t0, t1, t2, t3;\n\t"
-        "sub.u32 t0, %4, %8;\n\tsub.u32 t1, %5, %8;\n\tsub.u32 t2, %6, %8;\n\tsub.u32 t3, %7, %8;\n\t"
-        "setp.le.u32 p0, t0, %9;\n\tsetp.le.u32 p1, t1, %9;\n\t"
-        "setp.le.u32 p2, t2, %9;\n\tsetp.le.u32 p3, t3, %9;\n\t"
-        "or.pred q, p0, p1;\n\tor.pred q, q, p2;\n\tor.pred q, q, p3;\n\t"
-        "vote.sync.any.pred q, q, 0xffffffff;\n\t"
-        "@!q bra.uni BR_SKIP;\n\t"
-        "@p0 add.u32 %0, %0, %4;\n\t@p1 add.u32 %1, %1, %5;\n\t"
-        "@p2 add.u32 %2, %2, %6;\n\t@p3 add.u32 %3, %3, %7;\n\t"
-        "BR_SKIP:\n\t}"
-        : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3])
-        : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(L.loi), "r"(L.wm1));
-}
-template <>
-__device__ __forceinline__ void branchy_row<false, 4>(uint32_t (&a)[4], const uint32_t (&u)[4], const Lanes& L)
-{
-    asm volatile(
-        "{\n\t.reg .pred p0, p1, p2, p3, q;\n\t.reg .b32 t0, t1, t2, t3;\n\t"
-        "mad.lo.u32 t0, %4, %10, %8;\n\tmad.lo.u32 t1, %5, %10, %8;\n\t"
-        "mad.lo.u32 t2, %6, %10, %8;\n\tmad.lo.u32 t3, %7, %10, %8;\n\t"
-        "setp.le.u32 p0, t0, %9;\n\tsetp.le.u32 p1, t1, %9;\n\t"
-        "setp.le.u32 p2, t2, %9;\n\tsetp.le.u32 p3, t3, %9;\n\t"
-        "or.pred q, p0, p1;\n\tor.pred q, q, p2;\n\tor.pred q, q, p3;\n\t"
-        "vote.sync.any.pred q, q, 0xffffffff;\n\t"
-        "@!q bra.uni BR_SKIP;\n\t"
-        "@p0 mad.lo.u32 %0, %4, %10, %0;\n\t@p1 mad.lo.u32 %1, %5, %10, %1;\n\t"
-        "@p2 mad.lo.u32 %2, %6, %10, %2;\n\t@p3 mad.lo.u32 %3, %7, %10, %3;\n\t"
-        "BR_SKIP:\n\t}"
-        : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3])
-        : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(L.negloi), "r"(L.wm1), "r"(L.one));
-}
-template <>
 __device__ __forceinline__ void branchy_row<true, 2>(uint32_t (&a)[2], const uint32_t (&u)[2], const Lanes& L)
 {
     asm volatile(
@@ -434,30 +431,6 @@ __device__ __forceinline__ void branchy_row<false, 2>(uint32_t (&a)[2], const ui
 #define GB_BR_SUB_FMA(t, u, LOI, NLOI, ONE) "mad.lo.u32 " t ", " u ", " ONE ", " NLOI ";\n\t"
 #define GB_BR_ADD_ALU(p, a, u, ONE) "@" p " add.u32 " a ", " a ", " u ";\n\t"
 #define GB_BR_ADD_FMA(p, a, u, ONE) "@" p " mad.lo.u32 " a ", " u ", " ONE ", " a ";\n\t"
-#define GB_BR_TWO_ROWS4(SUBA, ADDA, SUBB, ADDB)                                                           \
-    asm volatile("{\n\t.reg .pred pa0, pa1, pa2, pa3, pb0, pb1, pb2, pb3, qa, qb;\n\t"                     \
-                 ".reg .b32 ta0, ta1, ta2, ta3, tb0, tb1, tb2, tb3;\n\t"                                  \
-                 SUBA("ta0", "%4", "%12", "%13", "%15") SUBA("ta1", "%5", "%12", "%13", "%15")            \
-                 SUBA("ta2", "%6", "%12", "%13", "%15") SUBA("ta3", "%7", "%12", "%13", "%15")            \
-                 SUBB("tb0", "%8", "%12", "%13", "%15") SUBB("tb1", "%9", "%12", "%13", "%15")            \
-                 SUBB("tb2", "%10", "%12", "%13", "%15") SUBB("tb3", "%11", "%12", "%13", "%15")          \
-                 "setp.le.u32 pa0, ta0, %14;\n\tsetp.le.u32 pa1, ta1, %14;\n\t"                           \
-                 "setp.le.u32 pa2, ta2, %14;\n\tsetp.le.u32 pa3, ta3, %14;\n\t"                           \
-                 "setp.le.u32 pb0, tb0, %14;\n\tsetp.le.u32 pb1, tb1, %14;\n\t"                           \
-                 "setp.le.u32 pb2, tb2, %14;\n\tsetp.le.u32 pb3, tb3, %14;\n\t"                           \
-                 "or.pred qa, pa0, pa1;\n\tor.pred qa, qa, pa2;\n\tor.pred qa, qa, pa3;\n\t"              \
-                 "or.pred qb, pb0, pb1;\n\tor.pred qb, qb, pb2;\n\tor.pred qb, qb, pb3;\n\t"              \
-                 "vote.sync.any.pred qa, qa, 0xffffffff;\n\tvote.sync.any.pred qb, qb, 0xffffffff;\n\t"  \
-                 "@!qa bra.uni BR_SKIP_A;\n\t"                                                            \
-                 ADDA("pa0", "%0", "%4", "%15") ADDA("pa1", "%1", "%5", "%15")                            \
-                 ADDA("pa2", "%2", "%6", "%15") ADDA("pa3", "%3", "%7", "%15")                            \
-                 "BR_SKIP_A:\n\t@!qb bra.uni BR_SKIP_B;\n\t"                                              \
-                 ADDB("pb0", "%0", "%8", "%15") ADDB("pb1", "%1", "%9", "%15")                            \
-                 ADDB("pb2", "%2", "%10", "%15") ADDB("pb3", "%3", "%11", "%15")                          \
-                 "BR_SKIP_B:\n\t}"                                                                        \
-                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3])                                         \
-                 : "r"(ua[0]), "r"(ua[1]), "r"(ua[2]), "r"(ua[3]), "r"(ub[0]), "r"(ub[1]), "r"(ub[2]),   \
-                   "r"(ub[3]), "r"(L.loi), "r"(L.negloi), "r"(L.wm1), "r"(L.one))
 #define GB_BR_TWO_ROWS2(SUBA, ADDA, SUBB, ADDB)                                                           \
     asm volatile("{\n\t.reg .pred pa0, pa1, pb0, pb1, qa, qb;\n\t.reg .b32 ta0, ta1, tb0, tb1;\n\t"       \
                  SUBA("ta0", "%2", "%6", "%7", "%9") SUBA("ta1", "%3", "%6", "%7", "%9")                  \
@@ -481,18 +454,11 @@ template <bool TOPA, bool TOPB, int LPT>
 __device__ __forceinline__ void branchy_two_rows(uint32_t (&a)[LPT], const uint32_t (&ua)[LPT],
                                                  const uint32_t (&ub)[LPT], const Lanes& L)
 {
-    if constexpr (LPT == 4) {
-        if constexpr (TOPA && TOPB) GB_BR_TWO_ROWS4(GB_BR_SUB_ALU, GB_BR_ADD_ALU, GB_BR_SUB_ALU, GB_BR_ADD_ALU);
-        else if constexpr (TOPA) GB_BR_TWO_ROWS4(GB_BR_SUB_ALU, GB_BR_ADD_ALU, GB_BR_SUB_FMA, GB_BR_ADD_FMA);
-        else if constexpr (TOPB) GB_BR_TWO_ROWS4(GB_BR_SUB_FMA, GB_BR_ADD_FMA, GB_BR_SUB_ALU, GB_BR_ADD_ALU);
-        else GB_BR_TWO_ROWS4(GB_BR_SUB_FMA, GB_BR_ADD_FMA, GB_BR_SUB_FMA, GB_BR_ADD_FMA);
-    } else {
-        static_assert(LPT == 2, "two-row blocks are written for 2 or 4 lanes per thread");
-        if constexpr (TOPA && TOPB) GB_BR_TWO_ROWS2(GB_BR_SUB_ALU, GB_BR_ADD_ALU, GB_BR_SUB_ALU, GB_BR_ADD_ALU);
-        else if constexpr (TOPA) GB_BR_TWO_ROWS2(GB_BR_SUB_ALU, GB_BR_ADD_ALU, GB_BR_SUB_FMA, GB_BR_ADD_FMA);
-        else if constexpr (TOPB) GB_BR_TWO_ROWS2(GB_BR_SUB_FMA, GB_BR_ADD_FMA, GB_BR_SUB_ALU, GB_BR_ADD_ALU);
-        else GB_BR_TWO_ROWS2(GB_BR_SUB_FMA, GB_BR_ADD_FMA, GB_BR_SUB_FMA, GB_BR_ADD_FMA);
-    }
+    static_assert(LPT == 2, "the PTX row votes are written for 2 lanes per thread");
+    if constexpr (TOPA && TOPB) GB_BR_TWO_ROWS2(GB_BR_SUB_ALU, GB_BR_ADD_ALU, GB_BR_SUB_ALU, GB_BR_ADD_ALU);
+    else if constexpr (TOPA) GB_BR_TWO_ROWS2(GB_BR_SUB_ALU, GB_BR_ADD_ALU, GB_BR_SUB_FMA, GB_BR_ADD_FMA);
+    else if constexpr (TOPB) GB_BR_TWO_ROWS2(GB_BR_SUB_FMA, GB_BR_ADD_FMA, GB_BR_SUB_ALU, GB_BR_ADD_ALU);
+    else GB_BR_TWO_ROWS2(GB_BR_SUB_FMA, GB_BR_ADD_FMA, GB_BR_SUB_FMA, GB_BR_ADD_FMA);
 }
 
 // One block, this thread's 4 lanes x 32 rows, every value valid.
@@ -509,21 +475,24 @@ __device__ __forceinline__ void branchy_two_rows(uint32_t (&a)[LPT], const uint3
 // vote.sync.any, one uniform branch around the predicated adds.  Which form is
 // faster depends on the width and on how many warps share an SM (the
 // autotuner picks per width).
-template <int B, bool BRANCHY, int ROWVOTE = 0, int LPT = default_lpt(B)>
+// In the row-major layout (LPT = 1) the thread's codes come from load_stream; the
+// decode is the same, all its shifts compile-time.
+template <int B, bool BRANCHY, int ROWVOTE = 0, int LPT = default_lpt(B), int LAY = kLayLanes>
 __device__ __forceinline__ void agg_block(const typename Geo<B, LPT>::Vec* rows, const Lanes& L,
                                           uint64_t& cnt, uint64_t& sum)
 {
     constexpr int kMode = B <= 21 ? 0 : (B <= 27 ? 1 : 2);
     constexpr int kLpt = LPT;
     typename Geo<B, LPT>::Vec W[B];
-    load_rows<B, LPT>(W, rows);
+    if constexpr (LAY == kLayLanes) load_rows<B, LPT>(W, rows);
+    else load_stream<B, LAY>(W, rows, threadIdx.x & 31);
     uint32_t a[kLpt] = {};
     uint32_t c = 0u;
     uint64_t s64 = 0u;
 #pragma unroll
     for (int r = 0; r < 32; ++r) {
         if constexpr (BRANCHY && ROWVOTE == 3) {
-            static_assert(kMode == 0 && (kLpt == 2 || kLpt == 4), "the PTX row vote is written for mode 0");
+            static_assert(kMode == 0 && kLpt == 2, "the PTX row vote is written for mode 0");
             if ((r & 1) == 0) {  // rows r and r + 1 (32 rows: always a pair)
                 uint32_t ua[kLpt], ub[kLpt];
 #pragma unroll
@@ -538,7 +507,7 @@ __device__ __forceinline__ void agg_block(const typename Geo<B, LPT>::Vec* rows,
                 else branchy_two_rows<false, false, kLpt>(a, ua, ub, L);
             }
         } else if constexpr (BRANCHY && ROWVOTE == 2) {
-            static_assert(kMode == 0 && (kLpt == 2 || kLpt == 4), "the PTX row vote is written for mode 0");
+            static_assert(kMode == 0 && kLpt == 2, "the PTX row vote is written for mode 0");
             uint32_t ui[kLpt];
 #pragma unroll
             for (int k = 0; k < kLpt; ++k) ui[k] = field_add<B, LPT>(W, r, k, L);
@@ -594,15 +563,15 @@ __device__ __forceinline__ void agg_block(const typename Geo<B, LPT>::Vec* rows,
                     if (top_field<B>(r)) acc1_alu(c, a[k], ui, L);
                     else if (sub_on_fma<B>(r, k)) acc1_fma(c, a[k], ui, L);
                     else acc1_imad(c, a[k], ui, L);
-                } else if constexpr (B < 32) {
+                } else if constexpr (B < 32 && LAY == kLayLanes) {
                     // 64-bit sums: count and sum on the FMA pipe (IMAD.WIDE); a
                     // top-of-word field (extracted by IMAD.HI) subtracts on the
                     // ALU.  At b = 28..31 this ran 1.5-6% faster than ALU adds.
                     if (top_field<B>(r)) acc2<true>(c, s64, ui, L);
                     else acc2<false>(c, s64, ui, L);
                 } else {
-                    // b = 32 (no extraction): plain compare and ALU adds, 2% faster
-                    // than the FMA form above
+                    // b = 32 (no extraction) and the row-major layout: plain compare and
+                    // ALU adds, 2-4% faster there than the FMA form above
                     if ((ui - L.loi) <= L.wm1) {
                         c += 1u;
                         s64 += ui;
@@ -693,137 +662,69 @@ __device__ __forceinline__ const typename Geo<B, LPT>::Vec* block_rows(const uns
 //   kLayLanes : lane-interleaved (strategy ii, everything above);
 //   kLayRow   : row-major bit stream, value j of the block at bits
 //               [j*b, j*b + b) of the block's 32*b words (strategy i);
-//   kLayBytes : b in {8, 16}: the codes as a plain uint8/uint16 array
-//               (strategy iii; b = 32 is the lane layout byte for byte).
-// The staging pipeline is shared; these consumers put all 32 lanes on one
-// block at a time, 32 codes per lane, with the accumulators of agg_block.
-enum Layout : int { kLayLanes = 0, kLayRow = 1, kLayBytes = 2 };
+// A byte-aligned array (strategy iii) is the row-major stream at b = 8 and 16, and
+// at b = 32 all three are the same bytes, so it needs no decoder of its own.
+// The order of a whole block's codes does not matter to COUNT and SUM, so a thread
+// may take any 32 codes of it that fill b whole words.
 
-template <int B, bool BRANCHY>
-__device__ __forceinline__ void acc_one(uint32_t ui, const Lanes& L, uint32_t& a, uint32_t& c, uint64_t& s64)
+// NB consecutive blocks, one lane's 32 codes of each: the blocks' independent
+// chains interleave.  Branchy: one vote for the blocks' 1024 * NB values, and the
+// sum (B selects and POPCs per block) is skipped when none matches.
+template <int B, bool BRANCHY, int LAY, int NB, typename Sum>
+__device__ __forceinline__ void agg_sliced(const uint32_t* words, int lane, const SliceKeys<B>& K, uint32_t& cnt,
+                                           Sum& sum)
 {
-    constexpr int kMode = B <= 21 ? 0 : (B <= 27 ? 1 : 2);
+    uint32_t X[NB][B], m[NB], any = 0u;
+#pragma unroll
+    for (int g = 0; g < NB; ++g) {
+        uint32_t W[B];
+        load_stream<B, LAY>(W, words + g * 32 * B, lane);
+        to_slices<B>(W, X[g], K.shift);
+        m[g] = slice_match<B>(X[g], K);
+        any |= m[g];
+    }
     if constexpr (BRANCHY) {
-        const uint32_t t = imad(ui, L.one, L.negloi);
-        const bool m = t <= L.wm1;
-        if (__any_sync(kFull, m)) {
-            if (m) {
-                if constexpr (kMode != 0) c += 1u;
-                if constexpr (kMode == 2) s64 += ui;
-                else a = imad(ui, L.one, a);
-            }
-        }
-    } else if constexpr (kMode == 0) {
-        acc0_fma(a, ui, L);  // subtract and add on the FMA pipe, one ISETP on the ALU
-    } else if constexpr (kMode == 1) {
-        acc1_imad(c, a, ui, L);
-    } else {
-        if ((ui - L.loi) <= L.wm1) {
-            c += 1u;
-            s64 += ui;
-        }
+        if (!__any_sync(kFull, any != 0u)) return;
+    }
+#pragma unroll
+    for (int g = 0; g < NB; ++g) {
+        cnt += static_cast<uint32_t>(__popc(m[g]));
+        sum += slice_sum<B>(X[g], m[g], K);
     }
 }
 
-// Fold one lane's 32 codes of accumulation into the 64-bit totals.
-template <int B>
-__device__ __forceinline__ void acc_flush(uint32_t a, uint32_t c, uint64_t s64, uint64_t& cnt, uint64_t& sum)
+// All `nb` (at most 64) blocks of a staged tile, bit-sliced.  A lane's partial
+// sums stay below 64 * 32 * 2^B, so up to B = 20 they are kept in 32 bits per tile.
+template <int B, bool BRANCHY, int LAY>
+__device__ __forceinline__ void scan_tile_sliced(const unsigned char* tile, uint32_t nb, int lane,
+                                                 const SliceKeys<B>& K, uint64_t& cnt, uint64_t& sum)
 {
-    constexpr int kMode = B <= 21 ? 0 : (B <= 27 ? 1 : 2);
-    if constexpr (kMode == 0) {
-        constexpr int kSB = (B + 5) & 31;
-        cnt += a >> kSB;
-        sum += a & ((1u << kSB) - 1u);
-    } else if constexpr (kMode == 1) {
-        cnt += c;
-        sum += a;
-    } else {
-        cnt += c;
-        sum += s64;
-    }
-}
-
-// Row-major block: lane l takes values j = l + 32m (m = 0..31), whose bits
-// start at l*B + 32*B*m: the word offset grows by B per m (an immediate) and
-// the shift (l*B) mod 32 is fixed per lane -- a variable-shift extractor, one
-// funnel shift over a two-word window per value.  The high word of the
-// block's last value lies one word past the block; it is read from shared
-// memory (the slot's neighbour) and contributes no bits.
-template <int B, bool BRANCHY>
-__device__ __forceinline__ void agg_block_row(const uint32_t* words, int lane, const Lanes& L, uint64_t& cnt,
-                                              uint64_t& sum)
-{
-    const uint32_t bit0 = static_cast<uint32_t>(lane) * B;
-    const uint32_t* w = words + (bit0 >> 5);
-    const uint32_t sh = bit0 & 31u;
-    uint32_t a = 0u, c = 0u;
-    uint64_t s64 = 0u;
-#pragma unroll
-    for (int m = 0; m < 32; ++m) {
-        uint32_t ui;
-        if constexpr (B == 32) {
-            ui = w[32 * m];
-        } else {
-            const uint32_t x = __funnelshift_r(w[B * m], w[B * m + 1], sh);
-            asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(ui) : "r"(x), "r"(L.mask), "r"(L.add));  // (x & mask) | add
-        }
-        acc_one<B, BRANCHY>(ui, L, a, c, s64);
-    }
-    acc_flush<B>(a, c, s64, cnt, sum);
-}
-
-// Byte-aligned block (B = 8 or 16): lane l reads the 16-byte chunks l and
-// l + 32 (B = 8) or l + 32h, h < 4 (B = 16); one byte permute per value
-// takes the code and ORs in the packed-count bit of L.add at once.
-template <int B, bool BRANCHY>
-__device__ __forceinline__ void agg_block_bytes(const unsigned char* blk, int lane, const Lanes& L,
-                                                uint64_t& cnt, uint64_t& sum)
-{
-    static_assert(B == 8 || B == 16, "byte-aligned widths are 8 and 16 (32 is the lane layout)");
-    const uint4* q4 = reinterpret_cast<const uint4*>(blk);
-    uint32_t a = 0u, c = 0u;
-    uint64_t s64 = 0u;
-#pragma unroll
-    for (int h = 0; h < B / 4; ++h) {
-        const uint4 q = q4[lane + 32 * h];
-        const uint32_t x[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-#pragma unroll
-            for (int k = 0; k < 32 / B; ++k) {
-                // B = 8 : bytes (x.k, add.1, add.0, add.0); add = 1 << 13 -> its byte 1 is 0x20
-                // B = 16: bytes (x.2k, x.2k+1, add.2, add.0); add = 1 << 21 -> its byte 2 is 0x20
-                constexpr unsigned kSel8 = 0x4450u;
-                constexpr unsigned kSel16 = 0x4600u;
-                const unsigned sel = B == 8 ? kSel8 + static_cast<unsigned>(k)
-                                            : kSel16 + static_cast<unsigned>(2 * k) +
-                                                  (static_cast<unsigned>(2 * k + 1) << 4);
-                const uint32_t ui = __byte_perm(x[e], L.add, sel);
-                acc_one<B, BRANCHY>(ui, L, a, c, s64);
-            }
-        }
-    }
-    acc_flush<B>(a, c, s64, cnt, sum);
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(tile);
+    uint32_t c = 0u, g = 0u;
+    typename std::conditional<(B <= 20), uint32_t, uint64_t>::type s = 0u;
+#pragma unroll 1
+    for (; g + 2u <= nb; g += 2u) agg_sliced<B, BRANCHY, LAY, 2>(words + g * 32u * B, lane, K, c, s);
+    if (g < nb) agg_sliced<B, BRANCHY, LAY, 1>(words + g * 32u * B, lane, K, c, s);
+    cnt += c;
+    sum += s;
 }
 
 // All `nb` blocks of a staged tile in a non-lane layout.
 template <int B, bool BRANCHY, int LAY>
-__device__ __forceinline__ void scan_tile_layout(const unsigned char* tile, uint32_t nb, int lane, const Lanes& L,
-                                                 uint64_t& cnt, uint64_t& sum)
+__device__ __forceinline__ void scan_tile_layout(const unsigned char* tile, uint32_t nb, int lane,
+                                                 const Keys<B, BRANCHY, LAY>& L, uint64_t& cnt, uint64_t& sum)
 {
-    constexpr uint32_t kBB = 128u * B;
-#pragma unroll 1
-    for (uint32_t g = 0; g < nb; ++g) {
-        if constexpr (LAY == kLayRow) {
-            agg_block_row<B, BRANCHY>(reinterpret_cast<const uint32_t*>(tile + g * kBB), lane, L, cnt, sum);
-        } else if constexpr (LAY == kLayBytes && (B == 8 || B == 16)) {
-            agg_block_bytes<B, BRANCHY>(tile + g * kBB, lane, L, cnt, sum);
-        }
+    if constexpr (sliced(B, BRANCHY, LAY)) {
+        scan_tile_sliced<B, BRANCHY, LAY>(tile, nb, lane, L, cnt, sum);
+    } else {
+#pragma unroll 2
+        for (uint32_t g = 0; g < nb; ++g)
+            agg_block<B, BRANCHY, 0, 1, LAY>(reinterpret_cast<const uint32_t*>(tile + g * (128u * B)), L, cnt, sum);
     }
 }
 
 // Tail block (n mod 1024 values) of a non-lane layout, from global memory.
-template <int B, int LAY>
+template <int B>
 __device__ __forceinline__ void scan_tail_layout(const ScanParams& p, int lane, uint64_t& cnt, uint64_t& sum)
 {
     const uint32_t* blk = p.packed + (p.n >> 10) * 32u * B;
@@ -832,11 +733,7 @@ __device__ __forceinline__ void scan_tail_layout(const ScanParams& p, int lane, 
     uint64_t s = 0u;
     for (uint32_t j = static_cast<uint32_t>(lane); j < rem; j += 32u) {
         uint32_t u;
-        if constexpr (LAY == kLayBytes && B == 8) {
-            u = reinterpret_cast<const uint8_t*>(blk)[j];
-        } else if constexpr (LAY == kLayBytes && B == 16) {
-            u = reinterpret_cast<const uint16_t*>(blk)[j];
-        } else if constexpr (B == 32) {
+        if constexpr (B == 32) {
             u = blk[j];
         } else {
             const uint32_t bit = j * B;
@@ -856,9 +753,13 @@ __device__ __forceinline__ void scan_tail_layout(const ScanParams& p, int lane, 
 // All `nb` blocks of a staged tile (blocks are contiguous in the slot).
 template <int B, bool BRANCHY, int ROWVOTE = 0, int LPT = default_lpt(B)>
 __device__ __forceinline__ void scan_tile(const unsigned char* tile, uint32_t nb, int lane,
-                                          const Lanes& L, uint32_t lo, uint32_t wm1, uint64_t& cnt,
+                                          const Keys<B, BRANCHY>& L, uint32_t lo, uint32_t wm1, uint64_t& cnt,
                                           uint64_t& sum)
 {
+    if constexpr (sliced(B, BRANCHY)) {
+        scan_tile_sliced<B, BRANCHY, kLayLanes>(tile, nb, lane, L, cnt, sum);
+        return;
+    } else {
     constexpr uint32_t kBB = 128u * B;
     constexpr uint32_t kStep = Geo<B, LPT>::kLpt;          // blocks per warp step
     const int q = lane % Geo<B, LPT>::kTpb;
@@ -871,6 +772,7 @@ __device__ __forceinline__ void scan_tile(const unsigned char* tile, uint32_t nb
         const bool ok = g + sub < nb;
         agg_block_masked<B, LPT>(block_rows<B, LPT>(tile + (ok ? g + sub : g) * kBB, q), lo, wm1, cnt, sum, ok,
                             1024u, q);
+    }
     }
 }
 
@@ -976,48 +878,51 @@ template <int B, bool BRANCHY, int LAY, int ROWVOTE, int LPT = default_lpt(B)>
 __device__ __forceinline__ bool walk_static(const ScanParams& p, const Pipe& P, int warp, int lane, int nwarps,
                                             uint64_t& cnt, uint64_t& sum)
 {
-    const uint64_t full_blocks = p.n >> 10;
-    const uint64_t ntiles = (full_blocks + P.tb - 1) / P.tb;
+    // a word of a power-of-two width holds whole codes in every layout, so the
+    // lane decode takes a row-major block as it is
+    constexpr int kDecode = slice_odd(B) == 1 ? static_cast<int>(kLayLanes) : LAY;
+    // n <= 2^31: block and tile numbers fit 32 bits
+    const uint32_t full_blocks = static_cast<uint32_t>(p.n >> 10);
+    const uint32_t ntiles = (full_blocks + P.tb - 1u) / P.tb;
+    const uint32_t last_nb = full_blocks - (ntiles - 1u) * P.tb;  // blocks of the last tile (ntiles > 0)
     // Warp-major numbering: a round's last, partial stretch of tiles goes to
     // warp slot w of every CTA before slot w + 1 of any, so the CTAs (SMs) of
     // a small column get equal shares (CTA-major numbering gave the first
     // CTAs two tiles per warp and the rest one at 2^24 values, b = 8).
-    const uint64_t gw = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;
-    const uint64_t GW = static_cast<uint64_t>(gridDim.x) * nwarps;
+    const uint32_t gw = static_cast<uint32_t>(warp) * gridDim.x + blockIdx.x;
+    const uint32_t GW = gridDim.x * static_cast<uint32_t>(nwarps);
 
-    auto issue = [&](uint64_t t, uint32_t s) {
-        const uint64_t fb = t * P.tb;
-        const uint64_t left = full_blocks - fb;
-        const uint32_t nb = left < P.tb ? static_cast<uint32_t>(left) : P.tb;
-        const uint32_t bytes = nb * (128u * B);
+    auto issue = [&](uint32_t t, uint32_t s) {
+        const uint32_t bytes = (t + 1u == ntiles ? last_nb : P.tb) * (128u * B);
         mbar_arrive_expect_tx(&P.bars[s], bytes);
-        bulk_g2s(P.slots + s * P.tile_bytes, p.packed + fb * 32u * B, bytes, &P.bars[s]);
+        bulk_g2s(P.slots + s * P.tile_bytes,
+                 reinterpret_cast<const unsigned char*>(p.packed) + static_cast<uint64_t>(t) * P.tile_bytes, bytes,
+                 &P.bars[s]);
     };
     if (lane == 0) {
         for (uint32_t s = 0; s < P.stages; ++s) {
-            const uint64_t t = gw + s * GW;
+            const uint32_t t = gw + s * GW;
             if (t < ntiles) issue(t, s);
         }
     }
 
-    const Lanes L = make_lanes<B>(p.lo, p.wm1);
+    const Keys<B, BRANCHY, kDecode> L = make_keys<B, BRANCHY, kDecode>(p.lo, p.wm1);
     uint32_t it = 0, s = 0, parity = 0;
     bool failed = false;
 #pragma unroll 1
-    for (uint64_t t = gw; t < ntiles; t += GW, ++it) {
+    for (uint32_t t = gw; t < ntiles; t += GW, ++it) {
         const bool ok = mbar_wait(&P.bars[s], parity, kWaitLimitNs);
         if (!__all_sync(kFull, ok)) {
             failed = true;
             break;
         }
-        const uint64_t left = full_blocks - t * P.tb;
-        const uint32_t nb = left < P.tb ? static_cast<uint32_t>(left) : P.tb;
-        if constexpr (LAY == kLayLanes)
+        const uint32_t nb = t + 1u == ntiles ? last_nb : P.tb;
+        if constexpr (kDecode == kLayLanes)
             scan_tile<B, BRANCHY, ROWVOTE, LPT>(P.slots + s * P.tile_bytes, nb, lane, L, p.lo, p.wm1, cnt, sum);
         else
-            scan_tile_layout<B, BRANCHY, LAY>(P.slots + s * P.tile_bytes, nb, lane, L, cnt, sum);
+            scan_tile_layout<B, BRANCHY, kDecode>(P.slots + s * P.tile_bytes, nb, lane, L, cnt, sum);
         __syncwarp();
-        const uint64_t tn = t + static_cast<uint64_t>(P.stages) * GW;
+        const uint32_t tn = t + P.stages * GW;
         if (lane == 0 && tn < ntiles) {
             fence_proxy_async_smem();
             issue(tn, s);
@@ -1031,9 +936,8 @@ __device__ __forceinline__ bool walk_static(const ScanParams& p, const Pipe& P, 
         if (lane == 0) atomicOr(p.status, kErrTimeout);
         // let copies still in flight land before the CTA's shared memory goes away
         for (uint32_t j = 0; j < P.stages; ++j) {
-            const uint64_t t = gw + static_cast<uint64_t>(it + j) * GW;
-            if (t >= ntiles) break;
             const uint32_t jt = it + j;
+            if (gw + jt * GW >= ntiles) break;
             mbar_wait(&P.bars[jt % P.stages], (jt / P.stages) & 1u, kDrainLimitNs);
         }
     }
@@ -1062,7 +966,7 @@ __global__ void __launch_bounds__(WMAX * 32, 1) k_scan_full(const ScanParams p)
         if constexpr (LAY == kLayLanes)
             scan_tail<B, LPT>(p, lane, cnt, sum);
         else
-            scan_tail_layout<B, LAY>(p, lane, cnt, sum);
+            scan_tail_layout<B>(p, lane, cnt, sum);
     }
     grid_finish<WMAX>(p, cnt, sum, false, (p.n + 1023u) >> 10);
 }
@@ -1242,7 +1146,7 @@ __global__ void __launch_bounds__(Shape<B>::kWarps * 32, 1) k_scan_queue(const S
     uint32_t next_id = 0;
     uint32_t next_nb = tn < ntiles ? ids_of(tn, next_id) : 0u;
 
-    const Lanes L = make_lanes<B>(p.lo, p.wm1);
+    const Keys<B, BRANCHY> L = make_keys<B, BRANCHY>(p.lo, p.wm1);
     uint64_t cnt = 0, sum = 0;
     uint32_t it = 0, s = 0, parity = 0;
     bool failed = false;
@@ -1302,10 +1206,8 @@ enum OpKind : int {
     kOpQueueBF = 2,
     kOpQueueBR = 3,
     kOpZoneBuild = 4,
-    kOpRowBF = 5,     // row-major layout (§3 strategy i)
+    kOpRowBF = 5,     // row-major layout (§3 strategy i) and byte arrays (iii), the same bytes
     kOpRowBR = 6,
-    kOpBytesBF = 7,   // byte-aligned layout, b = 8 or 16 (§3 strategy iii)
-    kOpBytesBR = 8,
     kOpBatchBF = 9,   // batched scans (one width group of a batch); only their shapes
     kOpBatchBR = 10,  // are kept here, the kernels live with the batch
 };
@@ -1327,6 +1229,27 @@ struct LaunchShape {
     int warps, stages, tile_blocks, vote_rows;
     int vec_lanes;  // lanes per thread and row (4 or 2; 0 = the width's default); full scans only
 };
+
+// Branchy full scans decoded directly whose per-value vote leaves them issue-bound
+// with 8 warps: their rule's shape is filled up to 16.  2^28 values, 8 warps of
+// 8 KB slots against 16 of one step, us: 112.9 / 95.4 at b = 17, 113.1 / 98.1 at 20,
+// 132.2 / 112.1 at 23, 131.2 / 127.1 at 25, 129.8 / 133.2 at 26, 159.9 / 134.4 at 28,
+// 160.0 / 144.4 at 30.
+__host__ __device__ constexpr bool branchy_filled(int b) { return !sliced(b, true) && (b <= 25 || b >= 28); }
+
+// Kernels compiled for CTAs of up to 16 warps fill up a shape of at most 8 warps:
+// as many as fit beside the slots, in whole fours (the SM has four schedulers: at
+// b = 16 14 warps took 89.4 us and 12 82.2), at most twice the shape's.
+inline LaunchShape filled(int b, LaunchShape s)
+{
+    if (s.warps <= 8) {
+        const int fit = static_cast<int>(static_cast<uint32_t>(kSmemMax) /
+                                         pipe_smem_bytes(static_cast<uint32_t>(b), 1, s.stages, s.tile_blocks));
+        const int most = fit < 2 * s.warps ? fit & ~3 : 2 * s.warps;
+        if (most > s.warps) s.warps = most;
+    }
+    return s;
+}
 
 template <int LO, int HI>
 __host__ inline ShapeInfo shape_range(int b)
