@@ -116,9 +116,8 @@ __device__ __forceinline__ CountSum batch_consume_body(const unsigned char* slot
     const uint32_t nfull = m.tail ? m.nk - 1u : m.nk;
     scan_tile<B, BRANCHY>(slot, nfull, lane, L, c.lo, c.wm1, cnt, sum);
     if (m.tail) {
-        const int q = lane % Geo<B>::kTpb;
-        agg_block_masked<B>(block_rows<B>(slot + nfull * (128u * B), q), c.lo, c.wm1, cnt, sum,
-                            lane < Geo<B>::kTpb, c.tail, q);
+        agg_block_masked<B, 1>(block_rows<B, 1>(slot + nfull * (128u * B), lane), c.lo, c.wm1, cnt, sum, true, c.tail,
+                               lane);
     }
     return CountSum{cnt, sum};
 }

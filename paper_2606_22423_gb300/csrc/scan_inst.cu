@@ -1,6 +1,7 @@
 // Instantiates the scan kernels for widths GB_BLO..GB_BHI (set by the build,
 // one object per range so the ranges compile in parallel) and exposes one
 // launcher per range.
+#include <algorithm>
 #include <atomic>
 
 #include "scan_kernels.cuh"
@@ -29,12 +30,36 @@ bool smem_configured()
     return true;
 }
 
-template <int B, auto KERNEL>
-cudaError_t launch_one(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
+// A full scan with at most one tile per warp of the full grid is cut finer, into
+// tiles of one warp step: on one CTA, whose sum needs no global round trip, while 16
+// warps hold it (n = 10^4: 2.0-2.7 us a launch against 4.7-5.7 on all SMs), then in
+// CTAs of 8 warps until they cover the SMs, then of as many as that takes.  (CTAs of
+// one warp: the last CTA's fold of their sums took a round trip per 32 of them.)
+inline void fit_small(const ScanParams& p, uint32_t step, LaunchShape& sh, int& grid)
+{
+    const uint64_t blocks = p.n >> 10;
+    const uint64_t sms = static_cast<uint64_t>(grid), most = static_cast<uint64_t>(sh.warps);
+    const uint64_t room = sms * most;
+    if (blocks > room * static_cast<uint64_t>(sh.tile_blocks)) return;
+    const uint64_t tb = std::max<uint64_t>(step, (blocks + room * step - 1) / (room * step) * step);
+    const uint64_t need = (blocks + tb - 1) / tb + ((p.n & 1023u) ? 1u : 0u);  // the tail takes a warp of its own
+    const uint64_t warps =
+        need <= most ? std::max<uint64_t>(need, 1u)
+                     : std::min<uint64_t>(std::max<uint64_t>((need + sms - 1) / sms, std::min<uint64_t>(8u, most)), most);
+    sh.tile_blocks = static_cast<int>(tb);
+    sh.stages = 1;
+    sh.warps = static_cast<int>(warps);
+    grid = static_cast<int>(std::min<uint64_t>((need + warps - 1) / warps, sms));
+    if (grid < 1) grid = 1;
+}
+
+template <int B, auto KERNEL, uint32_t SMALL_STEP = 0>
+cudaError_t launch_one(const ScanParams& p, LaunchShape sh, int grid, cudaStream_t st)
 {
     if (!smem_configured<KERNEL>())
         return cudaGetLastError() != cudaSuccess ? cudaGetLastError() : cudaErrorInvalidValue;
     ScanParams q = p;
+    if constexpr (SMALL_STEP != 0) fit_small(p, SMALL_STEP, sh, grid);
     q.tile_blocks = static_cast<uint32_t>(sh.tile_blocks);
     q.stages = static_cast<uint32_t>(sh.stages);
     const uint32_t smem = pipe_smem_bytes(B, sh.warps, sh.stages, sh.tile_blocks);
@@ -50,27 +75,28 @@ template <int B, bool BRANCHY>
 cudaError_t launch_full(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
 {
     if constexpr (sliced(B, BRANCHY)) {
-        return launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16>>(p, filled(B, sh), grid, st);
+        return launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16>, 1>(p, filled(B, sh), grid, st);
     } else {
+        constexpr uint32_t kStep = default_lpt(B);
         if constexpr (!BRANCHY && B <= 16) {  // the 2-lane geometry: 16-warp bound only
-            if (sh.vec_lanes == 2) return launch_one<B, k_scan_full<B, false, kLayLanes, 16, 0, 2>>(p, sh, grid, st);
+            if (sh.vec_lanes == 2) return launch_one<B, k_scan_full<B, false, kLayLanes, 16, 0, 2>, 2>(p, sh, grid, st);
         }
         if (sh.vec_lanes != 0 && sh.vec_lanes != default_lpt(B)) return cudaErrorInvalidValue;
         const bool w16 = sh.warps > 8;
         if constexpr (BRANCHY && B <= 21) {
             // the PTX row vote: the 16-warp bound only (any CTA up to 16 warps)
-            if (sh.vote_rows == 3) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 3>>(p, sh, grid, st);
-            if (sh.vote_rows == 2) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 2>>(p, sh, grid, st);
+            if (sh.vote_rows == 3) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 3>, kStep>(p, sh, grid, st);
+            if (sh.vote_rows == 2) return launch_one<B, k_scan_full<B, true, kLayLanes, 16, 2>, kStep>(p, sh, grid, st);
             if (sh.vote_rows)
-                return w16 ? launch_one<B, k_scan_full<B, true, kLayLanes, 16, 1>>(p, sh, grid, st)
-                           : launch_one<B, k_scan_full<B, true, kLayLanes, 8, 1>>(p, sh, grid, st);
+                return w16 ? launch_one<B, k_scan_full<B, true, kLayLanes, 16, 1>, kStep>(p, sh, grid, st)
+                           : launch_one<B, k_scan_full<B, true, kLayLanes, 8, 1>, kStep>(p, sh, grid, st);
         }
         if constexpr (BRANCHY && branchy_filled(B)) {
             const LaunchShape f = filled(B, sh);
-            if (f.warps > 8) return launch_one<B, k_scan_full<B, true, kLayLanes, 16>>(p, f, grid, st);
+            if (f.warps > 8) return launch_one<B, k_scan_full<B, true, kLayLanes, 16>, kStep>(p, f, grid, st);
         }
-        return w16 ? launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16>>(p, sh, grid, st)
-                   : launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 8>>(p, sh, grid, st);
+        return w16 ? launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 16>, kStep>(p, sh, grid, st)
+                   : launch_one<B, k_scan_full<B, BRANCHY, kLayLanes, 8>, kStep>(p, sh, grid, st);
     }
 }
 
@@ -79,9 +105,9 @@ template <int B, bool BRANCHY>
 cudaError_t launch_row(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
 {
     if constexpr (sliced(B, BRANCHY, row_decode(B)) || BRANCHY)
-        return launch_one<B, k_scan_full<B, BRANCHY, kLayRow, 16>>(p, filled(B, sh), grid, st);
+        return launch_one<B, k_scan_full<B, BRANCHY, kLayRow, 16>, 1>(p, filled(B, sh), grid, st);
     else
-        return launch_one<B, k_scan_full<B, BRANCHY, kLayRow>>(p, sh, grid, st);
+        return launch_one<B, k_scan_full<B, BRANCHY, kLayRow>, 1>(p, sh, grid, st);
 }
 
 template <int B>

@@ -731,7 +731,10 @@ __device__ __forceinline__ void scan_tail_layout(const ScanParams& p, int lane, 
     const uint32_t rem = static_cast<uint32_t>(p.n & 1023u);
     uint32_t c = 0u;
     uint64_t s = 0u;
-    for (uint32_t j = static_cast<uint32_t>(lane); j < rem; j += 32u) {
+#pragma unroll 8  // eight values' loads in flight
+    for (uint32_t m = 0; m < 32u; ++m) {
+        const uint32_t j = static_cast<uint32_t>(lane) + 32u * m;
+        if (j >= rem) continue;
         uint32_t u;
         if constexpr (B == 32) {
             u = blk[j];
@@ -777,10 +780,22 @@ __device__ __forceinline__ void scan_tile(const unsigned char* tile, uint32_t nb
 }
 
 // --------------------------------------------------------- grid reduction
+// Takes a ticket: everything this CTA wrote before it (its threads' writes
+// ordered by the barrier before) is visible to whoever reads the ticket after
+// it.  One acquire-release atomic; the full fences it replaces
+// cost a small scan about a microsecond.
+__device__ __forceinline__ unsigned int take_ticket(unsigned int* done)
+{
+    unsigned int t;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(done) : "memory");
+    return t;
+}
+
 // Sum (count, sum) over the grid: warp shuffles, one word pair per CTA, and
 // the last CTA to arrive folds the pairs, applies the frame of reference
-// (SUM_v = SUM_u + base*COUNT) and resets the ticket for the next launch.
-// WMAX bounds the CTA's warps (blockDim.x / 32 at run time).
+// (SUM_v = SUM_u + base*COUNT) and resets the ticket for the next launch.  A grid
+// of one CTA has nothing to fold.  WMAX bounds the CTA's warps (blockDim.x / 32 at
+// run time).
 template <int WMAX>
 __device__ __forceinline__ void grid_finish(const ScanParams& p, uint64_t cnt, uint64_t sum,
                                             bool queue_mode, uint64_t full_blocks_scanned)
@@ -799,74 +814,75 @@ __device__ __forceinline__ void grid_finish(const ScanParams& p, uint64_t cnt, u
         red[warp][1] = sum;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long c = 0, s = 0;
+    unsigned long long c = 0, s = 0;
+    if (threadIdx.x == 0)
         for (int w = 0; w < WARPS; ++w) {
             c += red[w][0];
             s += red[w][1];
         }
-        p.partials[2 * blockIdx.x] = c;
-        p.partials[2 * blockIdx.x + 1] = s;
-        __threadfence();
-        const unsigned t = atomicAdd(p.done, 1u);
-        is_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    unsigned long long c = 0, s = 0;
-    for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
-        c += __ldcg(&p.partials[2 * i]);
-        s += __ldcg(&p.partials[2 * i + 1]);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        c += __shfl_xor_sync(kFull, c, o);
-        s += __shfl_xor_sync(kFull, s, o);
-    }
-    __syncthreads();
-    if (lane == 0) {
-        red[warp][0] = c;
-        red[warp][1] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long tc = 0, ts = 0;
-        for (int w = 0; w < WARPS; ++w) {
-            tc += red[w][0];
-            ts += red[w][1];
+    if (gridDim.x > 1 || queue_mode) {
+        if (threadIdx.x == 0) {
+            p.partials[2 * blockIdx.x] = c;
+            p.partials[2 * blockIdx.x + 1] = s;
+            is_last = (take_ticket(p.done) == gridDim.x - 1);
         }
+        __syncthreads();
+        if (!is_last) return;
+        c = 0;
+        s = 0;
+        for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
+            c += __ldcg(&p.partials[2 * i]);
+            s += __ldcg(&p.partials[2 * i + 1]);
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            c += __shfl_xor_sync(kFull, c, o);
+            s += __shfl_xor_sync(kFull, s, o);
+        }
+        if (lane == 0) {
+            red[warp][0] = c;
+            red[warp][1] = s;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            c = 0;
+            s = 0;
+            for (int w = 0; w < WARPS; ++w) {
+                c += red[w][0];
+                s += red[w][1];
+            }
+        }
+    }
+    if (threadIdx.x == 0) {
         unsigned long long blocks = full_blocks_scanned;
         if (queue_mode) {
             blocks = __ldcg(&p.qctl[0]) + __ldcg(&p.qctl[2]);
-            tc += __ldcg(&p.qctl[3]);  // wholly-inside blocks answered from metadata
-            ts += __ldcg(&p.qctl[4]);
+            c += __ldcg(&p.qctl[3]);  // wholly-inside blocks answered from metadata
+            s += __ldcg(&p.qctl[4]);
             p.qctl[0] = 0ull;
             p.qctl[1] = 0ull;
             p.qctl[2] = 0ull;
             p.qctl[3] = 0ull;
             p.qctl[4] = 0ull;
         }
-        p.result[0] = static_cast<long long>(tc);
-        p.result[1] = static_cast<long long>(ts + static_cast<unsigned long long>(p.base) * tc);
+        p.result[0] = static_cast<long long>(c);
+        p.result[1] = static_cast<long long>(s + static_cast<unsigned long long>(p.base) * c);
         p.result[2] = static_cast<long long>(blocks);
         p.result[3] = 0;
-        __threadfence();
         *p.done = 0u;
     }
 }
 
-// Tail block (n mod 1024 values, zero padded) read straight from global memory.
-template <int B, int LPT = default_lpt(B)>
+// Tail block (n mod 1024 values, zero padded) read straight from global memory, a
+// lane per thread.
+template <int B>
 __device__ __forceinline__ void scan_tail(const ScanParams& p, int lane, uint64_t& cnt,
                                           uint64_t& sum)
 {
     const uint64_t tb = p.n >> 10;
     const uint32_t rem = static_cast<uint32_t>(p.n & 1023u);
-    const int q = lane % Geo<B, LPT>::kTpb;
-    const bool ok = lane < Geo<B, LPT>::kTpb;
-    const auto* rows = block_rows<B, LPT>(reinterpret_cast<const unsigned char*>(p.packed + tb * 32u * B), q);
-    agg_block_masked<B, LPT>(rows, p.lo, p.wm1, cnt, sum, ok, rem, q);
+    const auto* rows = block_rows<B, 1>(reinterpret_cast<const unsigned char*>(p.packed + tb * 32u * B), lane);
+    agg_block_masked<B, 1>(rows, p.lo, p.wm1, cnt, sum, true, rem, lane);
 }
 
 // ------------------------------------------------------------- full scan
@@ -964,7 +980,7 @@ __global__ void __launch_bounds__(WMAX * 32, 1) k_scan_full(const ScanParams p)
     const uint64_t gw = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;
     if ((p.n & 1023u) && gw == static_cast<uint64_t>(gridDim.x) * nwarps - 1) {
         if constexpr (LAY == kLayLanes)
-            scan_tail<B, LPT>(p, lane, cnt, sum);
+            scan_tail<B>(p, lane, cnt, sum);
         else
             scan_tail_layout<B>(p, lane, cnt, sum);
     }
