@@ -287,71 +287,6 @@ cudaError_t gb_column_select_ws(scan_column* c, uint64_t words, cudaStream_t st,
 // ---------------------------------------------------------------- encoders
 namespace {
 
-__global__ void k_encode(const uint32_t* __restrict__ v, uint64_t n, uint32_t b, uint32_t base,
-                         uint32_t* __restrict__ out, uint64_t words, unsigned int* status)
-{
-    // one thread per output word (block k, lane word w, lane l); the 32 lanes
-    // of a warp read 32 consecutive values per row and write 32 consecutive words
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-    const uint64_t span = 32ull * b;
-    const uint64_t mask = (b == 32) ? 0xffffffffull : ((1ull << b) - 1ull);
-    for (uint64_t t = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < words; t += stride) {
-        const uint64_t k = t / span;
-        const uint32_t rem = static_cast<uint32_t>(t - k * span);
-        const uint32_t w = rem >> 5, l = rem & 31u;
-        const uint32_t bit0 = 32u * w;                     // first stream bit of this word
-        const uint32_t r_first = bit0 / b;
-        const uint32_t r_last = min(31u, (bit0 + 31u) / b);
-        uint64_t acc = 0;
-        bool bad = false;
-        for (uint32_t r = r_first; r <= r_last; ++r) {
-            const uint64_t j = (k << 10) + 32ull * r + l;
-            uint64_t u = 0;
-            if (j < n) {
-                const uint32_t x = v[j];
-                u = static_cast<uint64_t>(x) - base;
-                // the thread holding the value's first bit checks its range
-                if (r * b >= bit0 && (x < base || (u & ~mask))) bad = true;
-                u &= mask;
-            }
-            const int64_t sh = static_cast<int64_t>(r) * b - bit0;
-            acc |= sh >= 0 ? (u << sh) : (u >> (-sh));
-        }
-        out[t] = static_cast<uint32_t>(acc);
-        if (bad) atomicOr(status, gb::kErrRange);
-    }
-}
-
-// Row-major stream (§3 strategy i; at b = 8/16/32 also the byte-aligned
-// array): one thread per output word; word t holds stream bits
-// [32t, 32t + 32), i.e. parts of values floor(32t/b) .. floor((32t+31)/b).
-__global__ void k_encode_rowmajor(const uint32_t* __restrict__ v, uint64_t n, uint32_t b, uint32_t base,
-                                  uint32_t* __restrict__ out, uint64_t words, unsigned int* status)
-{
-    const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-    const uint64_t mask = (b == 32) ? 0xffffffffull : ((1ull << b) - 1ull);
-    for (uint64_t t = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < words; t += stride) {
-        const uint64_t bit0 = 32ull * t;
-        const uint64_t first = bit0 / b, last = (bit0 + 31u) / b;
-        uint64_t acc = 0;
-        bool bad = false;
-        for (uint64_t j = first; j <= last; ++j) {
-            uint64_t u = 0;
-            if (j < n) {
-                const uint32_t x = v[j];
-                u = static_cast<uint64_t>(x) - base;
-                // the thread holding the value's first bit checks its range
-                if (j * b >= bit0 && (x < base || (u & ~mask))) bad = true;
-                u &= mask;
-            }
-            const int64_t sh = static_cast<int64_t>(j * b) - static_cast<int64_t>(bit0);
-            acc |= sh >= 0 ? (u << sh) : (u >> (-sh));
-        }
-        out[t] = static_cast<uint32_t>(acc);
-        if (bad) atomicOr(status, gb::kErrRange);
-    }
-}
-
 // Waits, with the library's bounded wait, on a transaction barrier that
 // nothing ever completes; the wait gives up after limit_ns and records the
 // timeout in the status word exactly as a lost copy would.
@@ -740,20 +675,11 @@ scan_status scan_encode_device_layout(const uint32_t* dev_values, uint64_t n, ui
     if (!dev_values || !dev_out) return fail(SCAN_EINVAL, "null pointer");
     if (reinterpret_cast<uintptr_t>(dev_out) & 15u) return fail(SCAN_EINVAL, "dev_out must be 16-byte aligned");
     cudaStream_t st = as_stream(stream);
-    unsigned int* flag = nullptr;
-    GB_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&flag), sizeof(unsigned int), st));
-    GB_CUDA(cudaMemsetAsync(flag, 0, sizeof(unsigned int), st));
-    const uint64_t words = scan_packed_words(n, b);
-    const int grid = persistent_grid() * 8;
-    if (layout == SCAN_LAYOUT_LANES)
-        k_encode<<<grid, 256, 0, st>>>(dev_values, n, b, base, dev_out, words, flag);
-    else
-        k_encode_rowmajor<<<grid, 256, 0, st>>>(dev_values, n, b, base, dev_out, words, flag);
-    GB_CUDA(cudaGetLastError());
+    // a byte array is the row-major stream's bytes
     unsigned int hflag = 0;
-    GB_CUDA(cudaMemcpyAsync(&hflag, flag, sizeof hflag, cudaMemcpyDeviceToHost, st));
-    GB_CUDA(cudaFreeAsync(flag, st));
-    GB_CUDA(cudaStreamSynchronize(st));
+    const cudaError_t e = gb_encode(static_cast<int>(b), layout != SCAN_LAYOUT_LANES, dev_values, n, base, dev_out, st,
+                                    &hflag);
+    if (e != cudaSuccess) return cuda_fail(e, "device encoder");
     if (hflag & gb::kErrRange) return fail(SCAN_EINVAL, "a value lies outside [base, base + 2^b)");
     return SCAN_OK;
 }

@@ -49,6 +49,10 @@ gb::LaunchShape gb_shape_for(int b, int op);
 std::vector<gb::LaunchShape> gb_shape_candidates(int b, int op);
 bool gb_shape_install(int b, int op, const gb::LaunchShape* shape, float tuned_us, float rule_us);
 
+// Runs the device encoder (n values to width b, lane layout or row-major) on st and
+// waits for it; *error gets kErrRange if a value lies outside [base, base + 2^b).
+cudaError_t gb_encode(int b, bool rowmajor, const uint32_t* values, uint64_t n, uint32_t base, uint32_t* out,
+                      cudaStream_t st, unsigned int* error);
 // Enqueues one scan of `c` (what scan_run_async does, with the result written
 // to dev_result); *empty is set when the predicate selects nothing and no
 // kernel was launched.
