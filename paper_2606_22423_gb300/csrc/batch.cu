@@ -49,18 +49,31 @@ int batch_grid() { return gb_device_sms(); }
 // then the status word at u32 index kMaxGroups.
 constexpr size_t kMaxGroups = 64;
 constexpr size_t kCtlWords = 40;  // u64 words: 64 + 1 u32 fit in 33
-constexpr int kBranches = 8;      // concurrent chains of width-group kernels in the graph
-constexpr int kPairChains = 2;    // chains 0 and 1: the large groups, narrow and wide widths
-// A group's time on the whole GPU by the bandwidth law, with GB300 figures
-// (copy bandwidth 6.7 TB/s, branch-free decode 4.3 Tvalues/s), in
+// A group's time on the whole GPU by the bandwidth law, with GB300 figures (copy
+// bandwidth 6.7 TB/s; 10 Tvalues/s of bit-sliced decode, 4.3 of direct), in
 // microseconds; its packed bytes and values count whole columns (zone skipping
 // only shortens it).
-double law_us(double bytes, int b) { return std::max(bytes / 6.7e6, bytes * 8.0 / b / 4.3e6); }
-// Groups shorter than this run on the small-group chains (2..7).
-constexpr double kSmallGroupUs = 16.0;
-// A group of this law time or more gets two CTAs per SM; a shorter one a
-// proportional share (fewer warps to start, to pop and to drain).
-constexpr double kFullGridUs = 10.0;
+double law_us(double bytes, int b)
+{
+    return std::max(bytes / 6.7e6, bytes * 8.0 / b / (gb::sliced(b, false) ? 10e6 : 4.3e6));
+}
+// The CTAs that start on a group are in proportion to its law time: two per SM for
+// `full` microseconds of it, which is the batch's own time over 1.5 -- so that one
+// wave and a half of CTAs hold the whole batch and each pays its ramp once -- and at
+// most kLongestUs, so that a large batch's later CTAs even out what zone maps and
+// the law get wrong.  1024 columns of 2^29 values in all (all widths), us per replay:
+// 261 / 248 / 248 / 256 / 274 for 1 / 1.5 / 2 / 4 / 6 waves; 2048 of 2^31: 859 / 782 /
+// 769 / 749 / 740; 64 of 2^26: 66 / 69 / 75 / 87 / 91.
+constexpr double kWaves = 1.5;
+constexpr double kLongestUs = 110.0;
+constexpr double kShortestUs = 5.0;
+// A pop is a share 1/(kPopPart * warps) of the group's work left, in units of a full
+// tile's time, of which starting a column (its descriptor, a short tile) costs
+// about kColumnCost: pops shrink towards the end, where the short columns are.
+// (Equal pops of a quarter of a warp's share: 11% slower on the same 1024 columns;
+// a least pop of 3 tiles instead of one: 4% slower.)
+constexpr double kPopPart = 2.0;
+constexpr double kColumnCost = 1.5;
 
 }  // namespace
 
@@ -71,49 +84,43 @@ struct scan_batch {
     std::vector<uint32_t> zone;        // 1 if the column skips by zone map
     std::vector<uint32_t> slot_of;     // index of the column in the descriptor table
     uint32_t ncol_k[2] = {0, 0};
-    uint32_t ntiles_k[2] = {0, 0};
-    uint32_t chunk_k[2] = {1, 1};
     uint32_t tiles_per_pop = 0;
     struct Group {
         int kernel, b;
         uint32_t first, count, ntiles, chunk;
-        int grid;
-        uint32_t chunk_off;  // offset of this group's chunk -> column table
+        int ctas;            // CTAs that start on this group
+        uint32_t chunk_off;  // offset of this group's pops in the chunk table
         gb::LaunchShape shape;  // warps, stages and tile blocks of this width group
         double bytes;           // packed bytes of its columns
     };
-    std::vector<Group> groups;  // one width-specialised launch each
-    uint32_t* d_chunk_col = nullptr;  // all groups' chunk -> first-column tables
+    std::vector<Group> groups;
+    struct Launch {  // groups of one flavour, range of widths, warps and stages
+        int kernel, warps, stages, grid;
+        std::vector<size_t> groups;
+    };
+    std::vector<Launch> launches;
+    uint2* d_chunks = nullptr;  // all groups' pops: first tile and column of each, one past the last
     size_t chunk_cap = 0;
     gb::BatchCol* h_table = nullptr;   // pinned
     gb::BatchCol* d_table = nullptr;
     unsigned long long* d_results = nullptr;  // 4 words per column, then 2 pop counters + status
     scan_result* h_results = nullptr;  // pinned copy of the results
     cudaStream_t capture_stream = nullptr;
-    cudaStream_t branch[kBranches] = {};  // capture-time branches (one graph node chain each)
-    cudaEvent_t fork = nullptr, join[kBranches] = {};
     cudaGraphExec_t graph = nullptr;
 };
 
-namespace gb {
-static cudaError_t launch_batch_kernel(bool branchy, int b, const BatchParams& p, int warps, int grid,
-                                       cudaStream_t st)
-{
-    return gb_launch_batch(branchy, b, p, warps, grid, st);
-}
-}  // namespace gb
-
 namespace {
 
-// Lay out the tiles for the current strategies: branch-free columns first,
-// and within each kernel by width, one width-specialised launch per group,
-// so that an SM runs at most two widths' decode code at a time (one CTA of
-// each graph chain; a kernel holding all 32 fully unrolled width variants
-// thrashed the instruction cache).
+// Lay out the tiles for the current strategies: branch-free columns first, and
+// within each flavour by width; the groups of four neighbouring widths that share a
+// shape's warps and stages go into one launch, whose CTAs each start on one of them,
+// so that an SM mostly runs one or two widths' decode code at a time (a kernel whose
+// warps all moved through 32 fully unrolled variants thrashed the instruction cache).
 scan_status layout(scan_batch* bt)
 {
     std::vector<uint32_t> order;
     std::vector<uint32_t> width(bt->ncols);
+    std::vector<uint64_t> length(bt->ncols);
     for (uint32_t i = 0; i < bt->ncols; ++i) {
         const uint2* zm = nullptr;
         const uint32_t* pk;
@@ -121,14 +128,21 @@ scan_status layout(scan_batch* bt)
         uint32_t b, base;
         gb_column_view(bt->cols[i], &pk, &n, &b, &base, &zm);
         width[i] = b;
+        length[i] = n;
     }
     for (int k = 0; k < 2; ++k)
         for (uint32_t b = 1; b <= 32; ++b)
+        {
+            const size_t first = order.size();
             for (uint32_t i = 0; i < bt->ncols; ++i)
                 if (bt->kernel_of[i] == k && width[i] == b) order.push_back(i);
+            // longest first: the short columns, whose starts cost a warp more than
+            // their few tiles, come last and in small pops
+            std::stable_sort(order.begin() + static_cast<std::ptrdiff_t>(first), order.end(),
+                             [&](uint32_t x, uint32_t y) { return length[x] > length[y]; });
+        }
     const size_t table_bytes = std::max<size_t>(1, bt->ncols) * sizeof(gb::BatchCol);
     std::memset(bt->h_table, 0, table_bytes);
-    uint32_t tiles[2] = {0, 0};
     bt->ncol_k[0] = bt->ncol_k[1] = 0;
     bt->groups.clear();
     uint32_t group_tiles = 0;
@@ -160,51 +174,80 @@ scan_status layout(scan_batch* bt)
         const uint64_t t = (nblocks + d.tile_blocks - 1) / d.tile_blocks;
         if (group_tiles + t > 0xffffffffull) return bfail(SCAN_EINVAL, "too many tiles in one batch");
         group_tiles += static_cast<uint32_t>(t);
-        tiles[k] += static_cast<uint32_t>(t);
         bt->groups.back().bytes += static_cast<double>(nblocks) * 128.0 * b;
         bt->groups.back().count += 1;
         bt->groups.back().ntiles = group_tiles;
         bt->slot_of[i] = j;
         bt->ncol_k[k] += 1;
     }
-    for (int k = 0; k < 2; ++k) bt->ntiles_k[k] = tiles[k];
     if (bt->groups.size() > kMaxGroups) return bfail(SCAN_EINVAL, "too many width groups");
-    // per group: two CTAs per SM for a group of kFullGridUs or more, a share
-    // in proportion to its law time below that (and a tile per warp at
-    // least), pops of about a quarter of a warp's share (at least 4 tiles),
-    // and a host-built table of each pop's first column.  Two CTAs per SM let
-    // the block scheduler give every SM one CTA of each concurrent chain; with
-    // one per SM the chains split the SMs between them and the replay took
-    // 22% longer.  Full grids for small groups cost 5-21% on batches of 64 and
-    // 512 columns (thousands of warps popping a few tiles from one counter).
-    std::vector<uint32_t> chunk_col;
+    std::vector<uint2> chunks;
     const uint64_t cap = 2ull * static_cast<uint64_t>(batch_grid());
-    for (auto& g : bt->groups) {
+    double total_us = 0.0;
+    for (const auto& g : bt->groups) total_us += law_us(g.bytes, g.b);
+    const double full_us = std::max(kShortestUs, std::min(kLongestUs, total_us / kWaves));
+    bt->launches.clear();
+    for (size_t gi = 0; gi < bt->groups.size(); ++gi) {
+        auto& g = bt->groups[gi];
         const uint64_t gw = static_cast<uint64_t>(g.shape.warps);
         const uint64_t by_tiles = (static_cast<uint64_t>(g.ntiles) + gw - 1) / gw;
         const uint64_t by_time =
-            static_cast<uint64_t>(std::ceil(static_cast<double>(cap) * law_us(g.bytes, g.b) / kFullGridUs));
-        g.grid = static_cast<int>(std::max<uint64_t>(1, std::min({by_tiles, by_time, cap})));
-        const uint32_t warps = static_cast<uint32_t>(g.grid * gw);
-        const uint32_t c = bt->tiles_per_pop ? bt->tiles_per_pop : std::max<uint32_t>(4, g.ntiles / (4 * warps));
-        g.chunk = std::min<uint32_t>(c, 1024);
-        g.chunk_off = static_cast<uint32_t>(chunk_col.size());
-        uint32_t col = g.first;
-        for (uint64_t t0 = 0; t0 < g.ntiles; t0 += g.chunk) {
-            while (col + 1 < g.first + g.count && bt->h_table[col + 1].tile_begin <= t0) ++col;
-            chunk_col.push_back(col - g.first);
+            static_cast<uint64_t>(std::ceil(static_cast<double>(cap) * law_us(g.bytes, g.b) / full_us));
+        g.ctas = static_cast<int>(std::max<uint64_t>(1, std::min({by_tiles, by_time, cap})));
+        if (g.ntiles) {
+            scan_batch::Launch* at = nullptr;
+            for (auto& l : bt->launches) {
+                const auto& h = bt->groups[l.groups.front()];
+                if (l.kernel == g.kernel && l.warps == g.shape.warps && l.stages == g.shape.stages &&
+                    (h.b - 1) / gb::kBatchRange == (g.b - 1) / gb::kBatchRange)
+                    at = &l;
+            }
+            if (!at) {
+                bt->launches.push_back({g.kernel, g.shape.warps, g.shape.stages, 0, {}});
+                at = &bt->launches.back();
+            }
+            at->groups.push_back(gi);
+            at->grid += g.ctas;
         }
+        const double warps = static_cast<double>(g.ctas) * static_cast<double>(gw);
+        double left = static_cast<double>(g.ntiles) + kColumnCost * g.count;
+        g.chunk_off = static_cast<uint32_t>(chunks.size());
+        uint32_t col = g.first, t = 0;
+        while (t < g.ntiles) {
+            while (col + 1 < g.first + g.count && bt->h_table[col + 1].tile_begin <= t) ++col;
+            chunks.push_back(make_uint2(t, col - g.first));
+            if (bt->tiles_per_pop) {
+                t = std::min(g.ntiles, t + bt->tiles_per_pop);
+                continue;
+            }
+            const double want = std::max(1.0, left / (kPopPart * warps));
+            double got = 0.0;
+            uint32_t c = col;
+            while (t < g.ntiles && got < want) {
+                if (bt->h_table[c].tile_begin == t) got += kColumnCost;
+                const uint32_t end = c + 1 < g.first + g.count ? bt->h_table[c + 1].tile_begin : g.ntiles;
+                const uint32_t take =
+                    std::max<uint32_t>(1, static_cast<uint32_t>(std::min<double>(end - t, std::ceil(want - got))));
+                const uint32_t n = std::min(take, end - t);
+                got += n;
+                t += n;
+                while (c + 1 < g.first + g.count && bt->h_table[c + 1].tile_begin <= t) ++c;
+            }
+            left -= got;
+        }
+        g.chunk = static_cast<uint32_t>(chunks.size()) - g.chunk_off;
+        chunks.push_back(make_uint2(g.ntiles, 0));
     }
-    if (chunk_col.size() > bt->chunk_cap) {
-        if (bt->d_chunk_col) cudaFree(bt->d_chunk_col);
-        bt->d_chunk_col = nullptr;
+    if (chunks.size() > bt->chunk_cap) {
+        if (bt->d_chunks) cudaFree(bt->d_chunks);
+        bt->d_chunks = nullptr;
         bt->chunk_cap = 0;
-        if (cudaMalloc(reinterpret_cast<void**>(&bt->d_chunk_col), chunk_col.size() * sizeof(uint32_t)) != cudaSuccess)
+        if (cudaMalloc(reinterpret_cast<void**>(&bt->d_chunks), chunks.size() * sizeof(uint2)) != cudaSuccess)
             return bfail(SCAN_ENOMEM, "chunk table allocation");
-        bt->chunk_cap = chunk_col.size();
+        bt->chunk_cap = chunks.size();
     }
-    if (!chunk_col.empty() &&
-        cudaMemcpy(bt->d_chunk_col, chunk_col.data(), chunk_col.size() * sizeof(uint32_t), cudaMemcpyHostToDevice) !=
+    if (!chunks.empty() &&
+        cudaMemcpy(bt->d_chunks, chunks.data(), chunks.size() * sizeof(uint2), cudaMemcpyHostToDevice) !=
             cudaSuccess)
         return bfail(SCAN_ECUDA, "chunk table upload");
     if (bt->graph) {
@@ -212,6 +255,34 @@ scan_status layout(scan_batch* bt)
         bt->graph = nullptr;
     }
     return SCAN_OK;
+}
+
+// Enqueues the kernel over `groups` (of one launch).
+cudaError_t launch_groups(scan_batch* bt, const std::vector<size_t>& groups, unsigned long long* ctl, cudaStream_t st)
+{
+    gb::BatchParams p{};
+    uint32_t ctas = 0, slot = 0;
+    for (const size_t gi : groups) {
+        const auto& g = bt->groups[gi];
+        gb::BatchGroup& d = p.g[p.ngroups++];
+        d.cols = bt->d_table + g.first;
+        d.chunks = bt->d_chunks + g.chunk_off;
+        d.head = reinterpret_cast<unsigned int*>(ctl) + gi;
+        d.b = static_cast<uint32_t>(g.b);
+        d.ncols = g.count;
+        d.ntiles = g.ntiles;
+        d.chunk = g.chunk;
+        d.slot_bytes = static_cast<uint32_t>(g.shape.tile_blocks) * 128u * d.b;
+        ctas += static_cast<uint32_t>(g.ctas);
+        d.cta_end = ctas;
+        slot = std::max(slot, d.slot_bytes);
+    }
+    const auto& g0 = bt->groups[groups.front()];
+    p.results = bt->d_results;
+    p.status = reinterpret_cast<unsigned int*>(ctl) + kMaxGroups;
+    p.stages = static_cast<uint32_t>(g0.shape.stages);
+    p.warp_bytes = p.stages * slot;
+    return gb_launch_batch(g0.kernel == 1, p, g0.shape.warps, static_cast<int>(ctas), st);
 }
 
 scan_status set_strategy(scan_batch* bt, uint32_t i, scan_strategy st)
@@ -456,11 +527,6 @@ scan_status scan_batch_create(scan_column* const* cols, uint32_t ncols, const sc
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&bt->d_results), res_bytes);
     if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&bt->h_results), res_bytes);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&bt->capture_stream, cudaStreamNonBlocking);
-    for (int k = 0; k < kBranches && e == cudaSuccess; ++k) {
-        e = cudaStreamCreateWithFlags(&bt->branch[k], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bt->join[k], cudaEventDisableTiming);
-    }
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bt->fork, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         scan_batch_destroy(bt);
         return bcuda(e, "batch allocation");
@@ -480,16 +546,11 @@ scan_status scan_batch_destroy(scan_batch* bt)
     cudaDeviceSynchronize();
     if (bt->graph) cudaGraphExecDestroy(bt->graph);
     if (bt->capture_stream) cudaStreamDestroy(bt->capture_stream);
-    for (int k = 0; k < kBranches; ++k) {
-        if (bt->branch[k]) cudaStreamDestroy(bt->branch[k]);
-        if (bt->join[k]) cudaEventDestroy(bt->join[k]);
-    }
-    if (bt->fork) cudaEventDestroy(bt->fork);
     if (bt->h_table) cudaFreeHost(bt->h_table);
     if (bt->h_results) cudaFreeHost(bt->h_results);
     if (bt->d_table) cudaFree(bt->d_table);
     if (bt->d_results) cudaFree(bt->d_results);
-    if (bt->d_chunk_col) cudaFree(bt->d_chunk_col);
+    if (bt->d_chunks) cudaFree(bt->d_chunks);
     delete bt;
     return SCAN_OK;
 }
@@ -567,68 +628,44 @@ scan_status scan_batch_exec(scan_batch* bt, const scan_pred* preds, void* stream
     const size_t res_words = 4ull * std::max<uint32_t>(1, bt->ncols) + kCtlWords;
     unsigned long long* ctl = bt->d_results + 4ull * std::max<uint32_t>(1, bt->ncols);
     if (!bt->graph) {
-        // copy descriptors -> reset -> {one kernel per width group, as parallel
-        // branches} -> copy results.  Branches let small groups run side by side
-        // and fill each other's tails; a group's grid is sized to its work.
+        // {copy descriptors, reset results and counters} -> the launches, side by
+        // side: captured on one stream whose dependencies are set by hand
         cudaStream_t cs = bt->capture_stream;
         BT_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        cudaMemcpyAsync(bt->d_table, bt->h_table, table_bytes, cudaMemcpyHostToDevice, cs);
-        cudaMemsetAsync(bt->d_results, 0, res_words * sizeof(unsigned long long), cs);
-        cudaEventRecord(bt->fork, cs);
-        // Large groups (law time kSmallGroupUs or more) on two chains: the
-        // narrow half in ascending width, the wide half in descending width,
-        // captured alternately.  At any moment a decode-bound kernel (small b)
-        // runs beside a bandwidth-bound one (large b), one CTA of each per SM,
-        // and both chains end on the middle widths.  (Eight chains in width
-        // order, one CTA per SM: 0.97 ms on the 4096-column workload; these two
-        // chains: 0.86-0.87 ms.  Halves cut by equal law time instead of equal
-        // group counts: 0.93 ms.)  Small groups, whose time is mostly launch
-        // and ramp, go round-robin on six more chains so that few of them queue
-        // behind one another: 512 columns of 2^28 values in all took 0.38 ms
-        // on the two chains and 0.23 ms this way.
-        std::vector<size_t> live, small;
-        for (size_t gi = 0; gi < bt->groups.size(); ++gi) {
-            const auto& g = bt->groups[gi];
-            if (!g.ntiles) continue;
-            (law_us(g.bytes, g.b) < kSmallGroupUs ? small : live).push_back(gi);
+        std::vector<cudaGraphNode_t> roots, ends;
+        cudaError_t ce = cudaSuccess;
+        const auto note = [&](std::vector<cudaGraphNode_t>& into) {  // the node captured last
+            cudaStreamCaptureStatus cst;
+            const cudaGraphNode_t* deps = nullptr;
+            size_t nd = 0;
+            if (ce == cudaSuccess) ce = cudaStreamGetCaptureInfo(cs, &cst, nullptr, nullptr, &deps, nullptr, &nd);
+            if (ce == cudaSuccess) into.insert(into.end(), deps, deps + nd);
+        };
+        const auto after = [&](std::vector<cudaGraphNode_t>& nodes) {  // what the next node waits for
+            if (ce == cudaSuccess)
+                ce = cudaStreamUpdateCaptureDependencies(cs, nodes.data(), nullptr, nodes.size(),
+                                                         cudaStreamSetCaptureDependencies);
+        };
+        ce = cudaMemcpyAsync(bt->d_table, bt->h_table, table_bytes, cudaMemcpyHostToDevice, cs);
+        note(roots);
+        std::vector<cudaGraphNode_t> none;
+        after(none);
+        if (ce == cudaSuccess) ce = cudaMemsetAsync(bt->d_results, 0, res_words * sizeof(unsigned long long), cs);
+        note(roots);
+        for (const auto& l : bt->launches) {
+            after(roots);
+            if (ce == cudaSuccess) ce = launch_groups(bt, l.groups, ctl, cs);
+            note(ends);
         }
-        const auto by_width = [&](size_t x, size_t y) { return bt->groups[x].b < bt->groups[y].b; };
-        std::stable_sort(live.begin(), live.end(), by_width);
-        std::stable_sort(small.begin(), small.end(), by_width);
-        const size_t half = (live.size() + 1) / 2;
-        std::vector<std::pair<size_t, int>> seq;  // (group, chain) in capture order
-        for (size_t i = 0; i < small.size(); ++i)
-            seq.push_back({small[i], kPairChains + static_cast<int>(i % (kBranches - kPairChains))});
-        for (size_t i = 0; i < half; ++i) {
-            seq.push_back({live[i], 0});
-            if (half + i < live.size()) seq.push_back({live[live.size() - 1 - i], 1});
-        }
-        bool used[kBranches] = {};
-        for (const auto& [gi, k] : seq) {
-            const auto& g = bt->groups[gi];
-            cudaStream_t bs = bt->branch[k];
-            if (!used[k]) cudaStreamWaitEvent(bs, bt->fork, 0);  // joins the capture
-            used[k] = true;
-            gb::BatchParams p{};
-            p.cols = bt->d_table + g.first;
-            p.chunk_col = bt->d_chunk_col + g.chunk_off;
-            p.ncols = g.count;
-            p.ntiles = g.ntiles;
-            p.chunk = g.chunk;
-            p.head = reinterpret_cast<unsigned int*>(ctl) + gi;
-            p.results = bt->d_results;
-            p.status = reinterpret_cast<unsigned int*>(ctl) + kMaxGroups;
-            p.stages = static_cast<uint32_t>(g.shape.stages);
-            p.slot_bytes = static_cast<uint32_t>(g.shape.tile_blocks) * 128u * static_cast<uint32_t>(g.b);
-            gb::launch_batch_kernel(g.kernel == 1, g.b, p, g.shape.warps, g.grid, bs);
-        }
-        for (int k = 0; k < kBranches; ++k) {
-            if (!used[k]) continue;
-            cudaEventRecord(bt->join[k], bt->branch[k]);
-            cudaStreamWaitEvent(cs, bt->join[k], 0);
-        }
+        if (!ends.empty()) after(ends);
+        else after(roots);
         cudaGraph_t g = nullptr;
-        const cudaError_t ec = cudaStreamEndCapture(cs, &g);
+        cudaError_t ec = cudaStreamEndCapture(cs, &g);
+        if (ec == cudaSuccess && ce != cudaSuccess) {
+            ec = ce;
+            if (g) cudaGraphDestroy(g);
+            g = nullptr;
+        }
         if (ec != cudaSuccess || !g) return bcuda(ec != cudaSuccess ? ec : cudaErrorUnknown, "graph capture");
         const cudaError_t ei = cudaGraphInstantiate(&bt->graph, g, 0);
         cudaGraphDestroy(g);
@@ -683,24 +720,14 @@ scan_status scan_batch_autotune(scan_batch* bt, const scan_pred* preds, uint32_t
         scan_status s = layout(bt);
         if (s != SCAN_OK) return s;
         fill_predicates(bt, preds);
-        const auto& g = bt->groups[gi];
         BT_CUDA(cudaMemcpyAsync(bt->d_table, bt->h_table, table_bytes, cudaMemcpyHostToDevice, st));
-        gb::BatchParams p{};
-        p.cols = bt->d_table + g.first;
-        p.chunk_col = bt->d_chunk_col + g.chunk_off;
-        p.ncols = g.count;
-        p.ntiles = g.ntiles;
-        p.chunk = g.chunk;
-        p.head = reinterpret_cast<unsigned int*>(ctl) + gi;
-        p.results = bt->d_results;
-        p.status = reinterpret_cast<unsigned int*>(ctl) + kMaxGroups;
-        p.stages = static_cast<uint32_t>(g.shape.stages);
-        p.slot_bytes = static_cast<uint32_t>(g.shape.tile_blocks) * 128u * static_cast<uint32_t>(g.b);
+        unsigned int* head = reinterpret_cast<unsigned int*>(ctl) + gi;
+        const std::vector<size_t> alone{gi};
         float total = 0.f;
         for (uint32_t r = 0; r <= reps; ++r) {  // the first launch warms up
-            BT_CUDA(cudaMemsetAsync(p.head, 0, sizeof(unsigned int), st));
+            BT_CUDA(cudaMemsetAsync(head, 0, sizeof(unsigned int), st));
             BT_CUDA(cudaEventRecord(e0, st));
-            BT_CUDA(gb::launch_batch_kernel(g.kernel == 1, g.b, p, g.shape.warps, g.grid, st));
+            BT_CUDA(launch_groups(bt, alone, ctl, st));
             BT_CUDA(cudaEventRecord(e1, st));
             BT_CUDA(cudaEventSynchronize(e1));
             float ms = 0.f;

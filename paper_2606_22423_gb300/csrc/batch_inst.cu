@@ -21,16 +21,24 @@ namespace {
 
 constexpr bool kBr = GB_BATCH_BRANCHY != 0;
 
-template <int BFIX>
-cudaError_t launch_fixed(const gb::BatchParams& p, int warps, int grid, cudaStream_t st)
+constexpr int kLo = GB_BLO;
+static_assert(GB_BHI - GB_BLO + 1 == gb::kBatchRange, "one kernel per range of four widths");
+
+}  // namespace
+
+// The groups' columns are all of widths GB_BLO..GB_BHI; CTAs of `warps` warps.
+cudaError_t GB_BATCH_LAUNCH(const gb::BatchParams& p, int warps, int grid, cudaStream_t st)
 {
-    if (warps < 1 || warps > 16) return cudaErrorInvalidValue;
+    if (warps < 1 || warps > 16 || p.ngroups < 1 || p.ngroups > static_cast<uint32_t>(gb::kBatchRange))
+        return cudaErrorInvalidValue;
+    for (uint32_t i = 0; i < p.ngroups; ++i)
+        if (p.g[i].b < static_cast<uint32_t>(GB_BLO) || p.g[i].b > static_cast<uint32_t>(GB_BHI)) return cudaErrorInvalidValue;
     static std::atomic<unsigned long long> configured{0ull};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
-    const void* fn = reinterpret_cast<const void*>(gb::k_scan_batch<kBr, BFIX>);
+    const void* fn = reinterpret_cast<const void*>(gb::k_scan_batch<kBr, kLo>);
     if (!(configured.load() & bit)) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, gb::kSmemMax);
         if (e != cudaSuccess) return e;
@@ -41,26 +49,8 @@ cudaError_t launch_fixed(const gb::BatchParams& p, int warps, int grid, cudaStre
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
-    const uint32_t smem = gb::batch_smem_bytes(static_cast<uint32_t>(warps), p.stages, p.slot_bytes);
-    gb::k_scan_batch<kBr, BFIX><<<grid, warps * 32, smem, st>>>(p);
+    const uint32_t smem =
+        static_cast<uint32_t>(warps) * (p.warp_bytes + p.stages * gb::kBatchSlotExtra);
+    gb::k_scan_batch<kBr, kLo><<<grid, warps * 32, smem, st>>>(p);
     return cudaGetLastError();
-}
-
-template <int LO, int HI>
-cudaError_t launch_width(int b, const gb::BatchParams& p, int warps, int grid, cudaStream_t st)
-{
-    if constexpr (LO > HI) {
-        return cudaErrorInvalidValue;
-    } else {
-        if (b == LO) return launch_fixed<LO>(p, warps, grid, st);
-        return launch_width<LO + 1, HI>(b, p, warps, grid, st);
-    }
-}
-
-}  // namespace
-
-// Columns all of width b (GB_BLO..GB_BHI), CTAs of `warps` warps.
-cudaError_t GB_BATCH_LAUNCH(int b, const gb::BatchParams& p, int warps, int grid, cudaStream_t st)
-{
-    return launch_width<GB_BLO, GB_BHI>(b, p, warps, grid, st);
 }

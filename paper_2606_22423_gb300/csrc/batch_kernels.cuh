@@ -34,17 +34,29 @@ struct BatchCol {
     uint32_t out;            // result slot
 };
 
-struct BatchParams {
+// One width group of a launch.
+struct BatchGroup {
     const BatchCol* cols;
-    const uint32_t* chunk_col;     // first column of every pop-sized chunk, or null (binary search)
+    const uint2* chunks;           // what each pop takes: first tile and its column, and one entry
+                                   // past the last; or null: `chunk` tiles per pop, column by search
+    unsigned int* head;            // pop counter, zero before the launch
+    uint32_t b;                    // width of every column
     uint32_t ncols;
     uint32_t ntiles;
-    uint32_t chunk;                // tiles per atomic pop
-    unsigned int* head;            // pop counter, zero before the launch
+    uint32_t chunk;                // entries of `chunks`, or tiles per pop without them
+    uint32_t slot_bytes;           // bytes per slot: the group's tile
+    uint32_t cta_end;              // CTAs below this number (and not below the group before's) start here
+};
+
+constexpr int kBatchRange = 4;     // widths per kernel, and groups per launch at most
+
+struct BatchParams {
+    BatchGroup g[kBatchRange];     // in any order of widths, all within the kernel's range
+    uint32_t ngroups;
     unsigned long long* results;   // per output slot: count, sum, blocks, 0
     unsigned int* status;
     uint32_t stages;               // slots per warp (warps per CTA = blockDim.x / 32)
-    uint32_t slot_bytes;           // bytes per slot: the group's largest tile
+    uint32_t warp_bytes;           // slot bytes per warp: stages of the launch's largest slot
 };
 
 // Default batch shape: 8 warps, each with 2 slots of 6 KB, and at most
@@ -89,111 +101,100 @@ __host__ __device__ constexpr int batch_default_warps(uint32_t b)
 }
 static_assert(batch_default_warps(32) == 6 && batch_default_warps(1) == 8, "default batch CTAs fit two per SM");
 
-struct SlotMeta {
-    uint32_t col;   // column index
-    uint32_t nk;    // blocks in the slot
-    uint32_t tail;  // 1 if the last block in the slot is the column's partial tail
-    uint32_t pad;
+struct __align__(8) SlotMeta {
+    uint32_t col;     // column index
+    uint32_t blocks;  // blocks in the slot, and kSlotTail if the last is the column's partial tail
 };
+constexpr uint32_t kSlotTail = 0x80000000u;
 
-struct CountSum {
-    uint64_t cnt, sum;
-};
-
-// The consumer's copy of its column's descriptor (what decoding a slot needs).
-struct ConsCol {
-    uint32_t lo, wm1;  // predicate in code space
-    uint32_t tail;     // values in the column's last block (0: whole)
-    uint32_t b;
-};
-
-template <int B, bool BRANCHY>
-__device__ __forceinline__ CountSum batch_consume_body(const unsigned char* slot, const SlotMeta m,
-                                                       const ConsCol& c, int lane)
-{
-    uint64_t cnt = 0, sum = 0;
-    const Keys<B, BRANCHY> L = make_keys<B, BRANCHY>(c.lo, c.wm1);
-    const uint32_t nfull = m.tail ? m.nk - 1u : m.nk;
-    scan_tile<B, BRANCHY>(slot, nfull, lane, L, c.lo, c.wm1, cnt, sum);
-    if (m.tail) {
-        agg_block_masked<B, 1>(block_rows<B, 1>(slot + nfull * (128u * B), lane), c.lo, c.wm1, cnt, sum, true, c.tail,
-                               lane);
-    }
-    return CountSum{cnt, sum};
-}
-
-// Every column of the launch has width BFIX and its decode is inlined: one
-// width's code per kernel keeps the instruction cache warm (a kernel holding
-// all 32 unrolled decoders stalled on instruction fetch), so a batch runs one
-// such kernel per width group.  Compiled for CTAs of up to 16 warps, which
-// caps it at 128 registers a thread: two 8-warp CTAs then fit one SM.
+// All tiles of one group that this warp pops.  One width's code at a time keeps the
+// instruction cache warm (warps popping tiles of all 32 widths stalled on
+// instruction fetch).  `phase` carries the slots' barrier parities from group to
+// group.  Returns false when a bounded wait gave up.
 template <bool BRANCHY, int BFIX>
-__global__ void __launch_bounds__(512, 1) k_scan_batch(const BatchParams P)
+__device__ __forceinline__ bool batch_group(const BatchGroup& P, unsigned long long* results, unsigned int* status,
+                                            int kStages, unsigned char* slots, uint64_t* bars, SlotMeta* meta,
+                                            uint32_t& phase, int lane)
 {
-    static_assert(BFIX >= 1 && BFIX <= 32, "batch kernels are width-specialised");
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t nwarps = blockDim.x >> 5;
-    const int kStages = static_cast<int>(P.stages);
     const uint32_t kSlot = P.slot_bytes;
-    unsigned char* slots = smem + static_cast<size_t>(warp) * kStages * kSlot;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(nwarps) * kStages * kSlot) +
-                     warp * kStages;
-    SlotMeta* meta =
-        reinterpret_cast<SlotMeta*>(smem + static_cast<size_t>(nwarps) * kStages * (kSlot + 8)) + warp * kStages;
-    if (lane == 0) {
-        for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
-        fence_mbar_init();
-    }
-    __syncwarp();
-
     // producer cursor (warp-uniform) and the descriptor of its column, kept in
     // registers: a warp's tiles come in runs of one column, so the descriptor
     // and the next column's first tile are loaded once per run, not per tile
+    const uint32_t tb = kSlot / (128u * BFIX);  // every column's tiles are cut alike
     uint32_t t_next = 0, t_end = 0, col = 0;
     bool exhausted = false;
-    uint32_t phase = 0;  // bit s: parity of slot s's next completion
     uint32_t pc_id = ~0u, next_begin = 0;
-    // zone skipping: blocks [zs_begin, zs_end) of column zs_col are known to hold no
-    // survivor (found by a look-ahead read of zone entries), so tiles inside
-    // that run are skipped without loading their entries again
-    uint32_t zs_col = ~0u;
-    uint64_t zs_begin = 0, zs_end = 0;
-    const uint32_t* pc_packed = nullptr;
+    uint32_t pc_begin = 0, pc_plain = 0, pc_flags = 0;  // tiles below pc_plain: full, copied whole
+    const unsigned char* pc_packed = nullptr;
     const uint2* pc_zm = nullptr;
     uint64_t pc_n = 0, pc_zlo = 0, pc_zhi = 0;
-    uint32_t pc_b = 0, pc_begin = 0, pc_tb = 0, pc_flags = 0;
+    // zone skipping: the keep bits of blocks [zw_begin, zw_begin + zw_span) of the
+    // column (one load of zone entries, a lane per block), and the next window's
+    // entries, loaded a window ahead
+    const uint32_t zw_span = tb <= 32u ? 32u / tb * tb : 0u;
+    uint32_t zw_begin = 0xffffffffu, zw_mask = 0u, zn_begin = 0xffffffffu;
+    uint2 zn = make_uint2(0u, 0u);
     auto load_col = [&](uint32_t c) {
         const BatchCol* d = P.cols + c;
-        pc_packed = d->packed;
+        pc_packed = reinterpret_cast<const unsigned char*>(d->packed);
         pc_zm = d->zonemap;
         pc_n = d->n;
-        pc_b = static_cast<uint32_t>(BFIX);
         pc_begin = d->tile_begin;
-        pc_tb = d->tile_blocks;
         pc_flags = d->flags;
         pc_zlo = d->zlo;
         pc_zhi = d->zhi;
         next_begin = c + 1 < P.ncols ? __ldg(&P.cols[c + 1].tile_begin) : 0xffffffffu;
+        pc_plain = pc_flags ? 0u : pc_begin + static_cast<uint32_t>(pc_n >> 10) / tb;
         pc_id = c;
+        zw_begin = 0xffffffffu;
+        zn_begin = 0xffffffffu;
+    };
+    const auto zone_entry = [&](uint32_t k, uint32_t nblocks) {
+        return k < nblocks ? __ldg(&pc_zm[k]) : make_uint2(0u, 0u);
+    };
+    const auto zone_keeps = [&](uint2 z) {
+        return static_cast<uint64_t>(z.y) >= pc_zlo && static_cast<uint64_t>(z.x) < pc_zhi;
+    };
+    // Keep bits of the nb (at most 64) blocks from k0.
+    auto zone_mask = [&](uint32_t k0, uint32_t nb, uint32_t nblocks) -> uint64_t {
+        if (nb > 32u || zw_span == 0u) {
+            const uint32_t lo = __ballot_sync(kFull, k0 + lane < nblocks && zone_keeps(zone_entry(k0 + lane, nblocks)));
+            const uint32_t k1 = k0 + 32u + static_cast<uint32_t>(lane);
+            const uint32_t hi = __ballot_sync(kFull, k1 < nblocks && zone_keeps(zone_entry(k1, nblocks)));
+            const uint64_t m = static_cast<uint64_t>(hi) << 32 | lo;
+            return nb >= 64u ? m : m & ((1ull << nb) - 1ull);
+        }
+        if (k0 < zw_begin || k0 + nb > zw_begin + zw_span || zw_begin == 0xffffffffu) {
+            const uint2 z = zn_begin == k0 ? zn : zone_entry(k0 + lane, nblocks);
+            zw_begin = k0;
+            zw_mask = __ballot_sync(kFull, k0 + lane < nblocks && zone_keeps(z));
+            zn_begin = k0 + zw_span;
+            zn = zone_entry(zn_begin + lane, nblocks);
+        }
+        const uint32_t m = zw_mask >> (k0 - zw_begin);
+        return nb >= 32u ? m : m & ((1u << nb) - 1u);
     };
 
-    // Next tile number, or false when the launch has no more work.
-    auto next_tile = [&](uint32_t& t) -> bool {
+    // Moves the cursor to a tile of the chunk, or to the next chunk; false when the
+    // group has no more work.
+    auto refill = [&]() -> bool {
         if (t_next >= t_end) {
             if (exhausted) return false;
             unsigned int start = 0;
-            if (lane == 0) start = atomicAdd(P.head, P.chunk);
+            if (lane == 0) start = atomicAdd(P.head, P.chunks ? 1u : P.chunk);
             start = __shfl_sync(kFull, start, 0);
-            if (start >= P.ntiles) {
+            if (start >= (P.chunks ? P.chunk : P.ntiles)) {
                 exhausted = true;
                 return false;
             }
-            t_next = start;
-            t_end = min(start + P.chunk, P.ntiles);
-            if (P.chunk_col) {  // host-built table: one load per pop
-                col = __ldg(&P.chunk_col[start / P.chunk]);
-            } else {            // binary search over tile_begin
+            if (P.chunks) {  // host-built table: one load per pop
+                const uint2 e = __ldg(&P.chunks[start]);
+                t_end = __ldg(&P.chunks[start + 1].x);
+                t_next = e.x;
+                col = e.y;
+            } else {         // binary search over tile_begin
+                t_next = start;
+                t_end = min(start + P.chunk, P.ntiles);
                 uint32_t lo = 0, hi = P.ncols - 1;
                 while (lo < hi) {
                     const uint32_t mid = (lo + hi + 1) >> 1;
@@ -204,68 +205,60 @@ __global__ void __launch_bounds__(512, 1) k_scan_batch(const BatchParams P)
             }
             if (col != pc_id) load_col(col);
         }
-        t = t_next++;
-        while (next_begin <= t) load_col(++col);  // the last column's next_begin is past every tile
+        while (next_begin <= t_next) load_col(++col);  // the last column's next_begin is past every tile
         return true;
     };
 
-    // Fetch the next tile into slot s; false when there is none.
+    // Fetch the next tile with a block to read into slot s; false when there is
+    // none.  Tiles without one (an empty predicate, no block kept by the zone map)
+    // are passed over, a whole run at a time.  meta[s]: the column and the blocks in
+    // the slot, the top bit set when the last of them is the column's partial tail.
     auto produce = [&](int s) -> bool {
-        uint32_t t;
-        if (!next_tile(t)) return false;
-        const uint32_t bb = 128u * pc_b;
-        const uint64_t nblocks = (pc_n + 1023u) >> 10;
-        const uint64_t k0 = static_cast<uint64_t>(t - pc_begin) * pc_tb;
-        const uint64_t left = nblocks - k0;
-        const uint32_t nb = left < pc_tb ? static_cast<uint32_t>(left) : pc_tb;
-        const bool has_tail = (pc_n & 1023u) && (k0 + nb == nblocks);
-        uint64_t keep = (nb >= 64) ? ~0ull : ((1ull << nb) - 1ull);
-        if (pc_flags & kColEmpty) {
-            keep = 0;
-        } else if (pc_flags & kColZone) {
-            if (zs_col == pc_id && k0 >= zs_begin && k0 + nb <= zs_end) {
-                keep = 0;  // inside a run already known to hold no survivor
-            } else if (nb < 32u) {
-                // one load covers this tile and the blocks after it, up to 32
-                const uint64_t span = nblocks - k0 < 32u ? nblocks - k0 : 32u;
-                bool k = false;
-                if (lane < span) {
-                    const uint2 z = __ldg(&pc_zm[k0 + lane]);
-                    k = static_cast<uint64_t>(z.y) >= pc_zlo && static_cast<uint64_t>(z.x) < pc_zhi;
-                }
-                const uint32_t m32 = __ballot_sync(kFull, k);
-                keep = m32 & ((1u << nb) - 1u);
-                if (!keep) {  // no survivor up to the first one found (or the whole span)
-                    zs_col = pc_id;
-                    zs_begin = k0;
-                    zs_end = k0 + (m32 ? static_cast<uint64_t>(__ffs(static_cast<int>(m32)) - 1) : span);
-                }
-            } else {
-                uint64_t km = 0;
-                for (uint32_t base_i = 0; base_i < nb; base_i += 32u) {
-                    const uint32_t i = base_i + lane;
-                    bool k = false;
-                    if (i < nb) {
-                        const uint2 z = __ldg(&pc_zm[k0 + i]);
-                        k = static_cast<uint64_t>(z.y) >= pc_zlo && static_cast<uint64_t>(z.x) < pc_zhi;
-                    }
-                    km |= static_cast<uint64_t>(__ballot_sync(kFull, k)) << base_i;
-                }
-                keep = km;
+        unsigned char* dst = slots + static_cast<uint32_t>(s) * kSlot;
+#pragma unroll 1
+        for (;;) {
+            if (t_next >= t_end || next_begin <= t_next) {
+                if (!refill()) return false;
             }
-        }
-        const uint32_t nk = static_cast<uint32_t>(__popcll(keep));
-        if (lane == 0) {
-            SlotMeta m;
-            m.col = col;
-            m.nk = nk;
-            m.tail = (has_tail && ((keep >> (nb - 1)) & 1ull)) ? 1u : 0u;
-            m.pad = 0;
-            meta[s] = m;
-            if (nk) {
+            const uint32_t t = t_next++;
+            if (t < pc_plain) {  // a whole tile, no zone test: one copy
+                if (lane == 0) {
+                    meta[s] = SlotMeta{col, tb};
+                    fence_proxy_async_smem();
+                    mbar_arrive_expect_tx(&bars[s], kSlot);
+                    bulk_g2s(dst, pc_packed + static_cast<uint64_t>(t - pc_begin) * kSlot, kSlot, &bars[s]);
+                }
+                __syncwarp();
+                return true;
+            }
+            if (pc_flags & kColEmpty) {
+                t_next = min(t_end, next_begin);
+                continue;
+            }
+            constexpr uint32_t bb = 128u * BFIX;
+            const uint32_t nblocks = static_cast<uint32_t>((pc_n + 1023u) >> 10);
+            const uint32_t k0 = (t - pc_begin) * tb;
+            const uint32_t nb = min(nblocks - k0, tb);
+            uint64_t keep = nb >= 64u ? ~0ull : (1ull << nb) - 1ull;
+            if (pc_flags & kColZone) {
+                keep = zone_mask(k0, nb, nblocks);
+                if (!keep) {
+                    // on to the tile of the window's next kept block, or past the window
+                    if (nb <= 32u && zw_span != 0u) {
+                        const uint32_t rest = zw_mask >> (k0 - zw_begin);
+                        const uint32_t run = rest ? static_cast<uint32_t>(__ffs(static_cast<int>(rest)) - 1)
+                                                  : zw_begin + zw_span - k0;
+                        t_next = min(min(t_end, next_begin), t + max(run / tb, 1u));
+                    }
+                    continue;
+                }
+            }
+            const uint32_t nk = static_cast<uint32_t>(__popcll(keep));
+            if (lane == 0) {
+                const bool tail = (pc_n & 1023u) && k0 + nb == nblocks && ((keep >> (nb - 1u)) & 1ull);
+                meta[s] = SlotMeta{col, nk | (tail ? kSlotTail : 0u)};
                 fence_proxy_async_smem();
                 mbar_arrive_expect_tx(&bars[s], nk * bb);
-                unsigned char* dst = slots + s * kSlot;
                 uint64_t rem = keep;
                 uint32_t placed = 0;
                 while (rem) {
@@ -273,14 +266,14 @@ __global__ void __launch_bounds__(512, 1) k_scan_batch(const BatchParams P)
                     const uint64_t from = rem >> first;
                     const uint32_t len = (~from == 0ull) ? (64u - first)
                                                           : static_cast<uint32_t>(__ffsll(static_cast<long long>(~from)) - 1);
-                    bulk_g2s(dst + placed * bb, pc_packed + (k0 + first) * 32u * pc_b, len * bb, &bars[s]);
+                    bulk_g2s(dst + placed * bb, pc_packed + static_cast<uint64_t>(k0 + first) * bb, len * bb, &bars[s]);
                     placed += len;
                     rem &= (len + first >= 64u) ? 0ull : (~0ull << (first + len));
                 }
             }
+            __syncwarp();
+            return true;
         }
-        __syncwarp();
-        return true;
     };
 
     int produced = 0;
@@ -291,7 +284,10 @@ __global__ void __launch_bounds__(512, 1) k_scan_batch(const BatchParams P)
 
     uint64_t cnt = 0, sum = 0, blocks = 0;
     int cur = -1;
-    ConsCol cc{0u, 0u, 0u, 0u};   // the consumer's column (loaded when it changes)
+    // the consumer's column, loaded when it changes; its keys too are made once per
+    // column (for a sliced width some 6 * b operations)
+    Keys<BFIX, BRANCHY> keys{};
+    uint32_t cc_lo = 0, cc_wm1 = 0, cc_tail = 0;
     uint32_t cur_out = 0, cur_base = 0;
     auto flush = [&]() {
         uint64_t c2 = cnt, s2 = sum;
@@ -301,7 +297,7 @@ __global__ void __launch_bounds__(512, 1) k_scan_batch(const BatchParams P)
             s2 += __shfl_xor_sync(kFull, s2, o);
         }
         if (lane == 0 && cur >= 0) {
-            unsigned long long* r = P.results + 4u * cur_out;
+            unsigned long long* r = results + 4u * cur_out;
             if (c2) atomicAdd(&r[0], static_cast<unsigned long long>(c2));
             if (c2) atomicAdd(&r[1], static_cast<unsigned long long>(s2 + static_cast<uint64_t>(cur_base) * c2));
             if (blocks) atomicAdd(&r[2], static_cast<unsigned long long>(blocks));
@@ -320,50 +316,90 @@ __global__ void __launch_bounds__(512, 1) k_scan_batch(const BatchParams P)
             flush();
             cur = static_cast<int>(m.col);
             const BatchCol* d = P.cols + m.col;
-            cc.lo = d->lo;
-            cc.wm1 = d->wm1;
-            cc.tail = static_cast<uint32_t>(d->n & 1023u);
-            cc.b = static_cast<uint32_t>(BFIX);
+            cc_lo = d->lo;
+            cc_wm1 = d->wm1;
+            cc_tail = static_cast<uint32_t>(d->n & 1023u);
+            keys = make_keys<BFIX, BRANCHY>(cc_lo, cc_wm1);
             cur_out = d->out;
             cur_base = d->base;
         }
-        if (m.nk) {
-            const bool ok = mbar_wait(&bars[s], (phase >> s) & 1u, kWaitLimitNs);
-            if (!__all_sync(kFull, ok)) {
-                failed = true;
-                break;
-            }
-            phase ^= 1u << s;
-            const CountSum r = batch_consume_body<BFIX, BRANCHY>(slots + s * kSlot, m, cc, lane);
-            cnt += r.cnt;
-            sum += r.sum;
-            blocks += m.nk;
+        const bool ok = mbar_wait(&bars[s], (phase >> s) & 1u, kWaitLimitNs);
+        if (!__all_sync(kFull, ok)) {
+            failed = true;
+            break;
         }
+        phase ^= 1u << s;
+        const unsigned char* slot = slots + static_cast<uint32_t>(s) * kSlot;
+        const uint32_t nk = m.blocks & ~kSlotTail;
+        const bool tail = (m.blocks & kSlotTail) != 0u;
+        const uint32_t nfull = tail ? nk - 1u : nk;
+        scan_tile<BFIX, BRANCHY>(slot, nfull, lane, keys, cc_lo, cc_wm1, cnt, sum);
+        if (tail)
+            agg_block_masked<BFIX, 1>(block_rows<BFIX, 1>(slot + nfull * (128u * BFIX), lane), cc_lo, cc_wm1, cnt,
+                                      sum, true, cc_tail, lane);
+        blocks += nk;
         __syncwarp();
         if (produce(s)) ++produced;
     }
     if (failed) {
-        if (lane == 0) atomicOr(P.status, kErrTimeout);
+        if (lane == 0) atomicOr(status, kErrTimeout);
         // let this warp's copies in flight land before shared memory is released
         for (int j = it; j < produced && j < it + kStages; ++j) {
             const int s = j % kStages;
-            if (meta[s].nk) {
-                mbar_wait(&bars[s], (phase >> s) & 1u, kDrainLimitNs);
-                phase ^= 1u << s;
-            }
+            mbar_wait(&bars[s], (phase >> s) & 1u, kDrainLimitNs);
+            phase ^= 1u << s;
         }
     }
     flush();
+    return !failed;
+}
+
+// A kernel serves a range of four widths.  Every CTA starts on one of the launch's
+// width groups (its share of the CTAs follows its law time) and its warps go on to
+// the next when that has no tile left, so that a group finished early -- zone maps
+// skipped most of it -- leaves no SM idle, and a batch of all 32 widths takes 8
+// launches side by side instead of 32 in chains (each of those cost some 12 us of
+// ramp and drain).  Compiled for CTAs of up to 16 warps, which caps it at 128
+// registers a thread: two 8-warp CTAs then fit one SM.
+template <bool BRANCHY, int LO>
+__global__ void __launch_bounds__(512, 1) k_scan_batch(const __grid_constant__ BatchParams P)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t nwarps = blockDim.x >> 5;
+    const int stages = static_cast<int>(P.stages);
+    unsigned char* slots = smem + static_cast<size_t>(warp) * P.warp_bytes;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(nwarps) * P.warp_bytes) + warp * stages;
+    SlotMeta* meta =
+        reinterpret_cast<SlotMeta*>(smem + static_cast<size_t>(nwarps) * (P.warp_bytes + 8u * P.stages)) + warp * stages;
+    if (lane == 0) {
+        for (int s = 0; s < stages; ++s) mbar_init(&bars[s], 1);
+        fence_mbar_init();
+    }
+    __syncwarp();
+    uint32_t first = 0;
+    while (first + 1 < P.ngroups && blockIdx.x >= P.g[first].cta_end) ++first;
+    uint32_t phase = 0;  // bit s: parity of slot s's next completion
+    bool ok = true;
+#pragma unroll 1
+    for (uint32_t i = 0; i < P.ngroups && ok; ++i) {
+        const BatchGroup& g = P.g[first + i < P.ngroups ? first + i : first + i - P.ngroups];
+        switch (static_cast<int>(g.b) - LO) {
+        case 0: ok = batch_group<BRANCHY, LO>(g, P.results, P.status, stages, slots, bars, meta, phase, lane); break;
+        case 1: ok = batch_group<BRANCHY, LO + 1>(g, P.results, P.status, stages, slots, bars, meta, phase, lane); break;
+        case 2: ok = batch_group<BRANCHY, LO + 2>(g, P.results, P.status, stages, slots, bars, meta, phase, lane); break;
+        case 3: ok = batch_group<BRANCHY, LO + 3>(g, P.results, P.status, stages, slots, bars, meta, phase, lane); break;
+        default: break;  // the host groups widths by range
+        }
+    }
 }
 
 }  // namespace gb
 
 // One launcher per flavour and range of four widths (separate objects).
 #define GB_DECLARE_BATCH(lo, hi)                                                                                \
-    cudaError_t gb_launch_batch_bf_##lo##_##hi##_w(int b, const gb::BatchParams& p, int warps, int grid,        \
-                                                   cudaStream_t st);                                             \
-    cudaError_t gb_launch_batch_br_##lo##_##hi##_w(int b, const gb::BatchParams& p, int warps, int grid,        \
-                                                   cudaStream_t st);
+    cudaError_t gb_launch_batch_bf_##lo##_##hi##_w(const gb::BatchParams& p, int warps, int grid, cudaStream_t st); \
+    cudaError_t gb_launch_batch_br_##lo##_##hi##_w(const gb::BatchParams& p, int warps, int grid, cudaStream_t st);
 GB_DECLARE_BATCH(1, 4)
 GB_DECLARE_BATCH(5, 8)
 GB_DECLARE_BATCH(9, 12)
@@ -374,15 +410,15 @@ GB_DECLARE_BATCH(25, 28)
 GB_DECLARE_BATCH(29, 32)
 #undef GB_DECLARE_BATCH
 
-// The batch kernel of one width group: flavour, width b, CTAs of `warps` warps.
-inline cudaError_t gb_launch_batch(bool branchy, int b, const gb::BatchParams& p, int warps, int grid,
-                                   cudaStream_t st)
+// The batch kernel over p's groups, all of one range of widths and of CTAs of
+// `warps` warps.
+inline cudaError_t gb_launch_batch(bool branchy, const gb::BatchParams& p, int warps, int grid, cudaStream_t st)
 {
 #define GB_RANGE(k, lo, hi)                                                                                       \
     case k:                                                                                                      \
-        return branchy ? gb_launch_batch_br_##lo##_##hi##_w(b, p, warps, grid, st)                                 \
-                       : gb_launch_batch_bf_##lo##_##hi##_w(b, p, warps, grid, st);
-    switch ((b - 1) / 4) {
+        return branchy ? gb_launch_batch_br_##lo##_##hi##_w(p, warps, grid, st)                                     \
+                       : gb_launch_batch_bf_##lo##_##hi##_w(p, warps, grid, st);
+    switch (static_cast<int>(p.g[0].b - 1) / gb::kBatchRange) {
         GB_RANGE(0, 1, 4)
         GB_RANGE(1, 5, 8)
         GB_RANGE(2, 9, 12)

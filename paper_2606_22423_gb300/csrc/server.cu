@@ -147,11 +147,14 @@ cudaError_t launch_slot(scan_server* sv, Slot& s, const char** step)
         if (!g.ntiles) continue;
         *step = "batch kernel launch";
         gb::BatchParams p{};
-        p.cols = s.d_tab + g.first;
-        p.ncols = g.count;
-        p.ntiles = g.ntiles;
-        p.chunk = std::max<uint32_t>(1, std::min<uint32_t>(256, g.ntiles / (8 * warps)));
-        p.head = ctl + gi;
+        p.ngroups = 1;
+        gb::BatchGroup& d = p.g[0];
+        d.cols = s.d_tab + g.first;
+        d.b = g.b;
+        d.ncols = g.count;
+        d.ntiles = g.ntiles;
+        d.chunk = std::max<uint32_t>(1, std::min<uint32_t>(256, g.ntiles / (8 * warps)));
+        d.head = ctl + gi;
         p.results = s.d_res;
         p.status = ctl + 33;
         // the default batch shape (the tiles were cut by batch_tile_blocks) and
@@ -161,8 +164,10 @@ cudaError_t launch_slot(scan_server* sv, Slot& s, const char** step)
         // and at 1.5x the queue grew (p50 37 ms) where it now serves every
         // query (p50 0.55 ms).
         p.stages = gb::kBatchStages;
-        p.slot_bytes = gb::batch_tile_blocks(g.b) * 128u * g.b;
-        e = gb_launch_batch(false, static_cast<int>(g.b), p, gb::batch_default_warps(g.b), 2 * sv->sms, s.stream);
+        d.slot_bytes = gb::batch_tile_blocks(g.b) * 128u * g.b;
+        p.warp_bytes = p.stages * d.slot_bytes;
+        d.cta_end = 2u * static_cast<uint32_t>(sv->sms);
+        e = gb_launch_batch(false, p, gb::batch_default_warps(g.b), 2 * sv->sms, s.stream);
     }
     if (e == cudaSuccess) {
         // results of the n entries, then the control words (pop counters, status)
