@@ -530,8 +530,9 @@ scan_status auto_survivors(scan_column* c, uint64_t zlo, uint64_t zhi, cudaStrea
     return SCAN_OK;
 }
 
+// The result goes to `result` (device or pinned host memory); extra_flags as ScanParams::flags.
 scan_status enqueue_scan(scan_column* c, scan_pred pred, scan_strategy strategy, cudaStream_t st,
-                         long long* dev_result, bool* empty)
+                         long long* result, bool* empty, uint32_t extra_flags = 0u)
 {
     gb::ScanParams p = base_params(c);
     *empty = false;
@@ -539,7 +540,8 @@ scan_status enqueue_scan(scan_column* c, scan_pred pred, scan_strategy strategy,
         *empty = true;
         return SCAN_OK;
     }
-    if (dev_result) p.result = dev_result;
+    p.result = result;
+    p.flags |= extra_flags;
     if (strategy == SCAN_AUTO) {
         strategy = SCAN_BRANCHFREE;
         if (c->zonemap_valid && c->layout == SCAN_LAYOUT_LANES) {
@@ -919,21 +921,21 @@ scan_status scan_run(scan_column* col, scan_pred pred, scan_strategy strategy, v
     if (!col || !host_out) return fail(SCAN_EINVAL, "null pointer");
     cudaStream_t st = as_stream(stream);
     bool empty = false;
-    scan_status s = enqueue_scan(col, pred, strategy, st, nullptr, &empty);
+    // the kernel writes the result, with the status word in its last one, to pinned host memory
+    scan_status s = enqueue_scan(col, pred, strategy, st, reinterpret_cast<long long*>(col->host_result), &empty,
+                                 gb::kFlagStatus);
     if (s != SCAN_OK) return s;
     if (empty) {
         std::memset(host_out, 0, sizeof *host_out);
         return SCAN_OK;
     }
-    // result (32 B) and status word (4 B) are adjacent: one small copy
-    GB_CUDA(cudaMemcpyAsync(col->host_result, col->ws.result, 36, cudaMemcpyDeviceToHost, st));
     GB_CUDA(cudaStreamSynchronize(st));
-    unsigned int dev_status = 0;
-    std::memcpy(&dev_status, reinterpret_cast<unsigned char*>(col->host_result) + 32, 4);
+    const unsigned int dev_status = static_cast<unsigned int>(col->host_result->reserved);
     if (dev_status) {
         GB_CUDA(cudaMemset(col->ws_raw, 0, Workspace::kBytes));
         return fail(SCAN_ETIMEOUT, "a device-side wait timed out (status 0x%x)", dev_status);
     }
+    col->host_result->reserved = 0;
     *host_out = *col->host_result;
     return SCAN_OK;
 }

@@ -26,7 +26,7 @@
 namespace gb {
 
 enum : uint32_t { kErrTimeout = 1u, kErrRange = 2u };
-enum : uint32_t { kFlagAgg = 1u };
+enum : uint32_t { kFlagAgg = 1u, kFlagStatus = 2u };
 
 struct ScanParams {
     const uint32_t* packed;       // lane-interleaved words, 16-byte aligned
@@ -34,7 +34,8 @@ struct ScanParams {
     uint32_t base;                // frame-of-reference base
     uint32_t lo;                  // predicate lower bound in code space
     uint32_t wm1;                 // predicate width minus one (width >= 1)
-    uint32_t flags;               // kFlagAgg: answer wholly-inside blocks from their metadata
+    uint32_t flags;               // kFlagAgg: answer wholly-inside blocks from their metadata;
+                                  // kFlagStatus: the result's last word gets the status word
     uint64_t zlo, zhi;            // predicate [zlo, zhi) on decoded values, for zone tests
     const uint2* zonemap;         // (min, max) of decoded values per block
     uint2* zonemap_out;           // zone-map build output
@@ -868,7 +869,8 @@ __device__ __forceinline__ void grid_finish(const ScanParams& p, uint64_t cnt, u
         p.result[0] = static_cast<long long>(c);
         p.result[1] = static_cast<long long>(s + static_cast<unsigned long long>(p.base) * c);
         p.result[2] = static_cast<long long>(blocks);
-        p.result[3] = 0;
+        // every CTA set its error bits before its ticket
+        p.result[3] = (p.flags & kFlagStatus) ? static_cast<long long>(__ldcg(p.status)) : 0;
         *p.done = 0u;
     }
 }
