@@ -57,9 +57,14 @@ struct Group {
     uint32_t b, first, count, ntiles;
 };
 
+constexpr int kSlotChains = 4;  // streams a slot's width kernels are spread over
+
 struct Slot {
     std::vector<Group> groups;
-    cudaStream_t stream = nullptr;
+    cudaStream_t stream = nullptr;                 // copies, and the first chain
+    cudaStream_t chain[kSlotChains - 1] = {};      // the other chains
+    cudaEvent_t ready = nullptr;                   // descriptors and counters in place
+    cudaEvent_t joined[kSlotChains - 1] = {};
     cudaEvent_t done = nullptr;
     gb::BatchCol* h_tab = nullptr;
     gb::BatchCol* d_tab = nullptr;
@@ -142,9 +147,20 @@ cudaError_t launch_slot(scan_server* sv, Slot& s, const char** step)
     }
     unsigned int* ctl = reinterpret_cast<unsigned int*>(s.d_res + 4ull * s.cap);
     const uint32_t warps = static_cast<uint32_t>(sv->sms) * gb::kBatchWarps;
+    // The width kernels go round the slot's chains: a small batch's kernels are
+    // mostly ramp and drain (a 2-query batch of 6 widths took 60 us one after the
+    // other), and a large one's fill each other's tails.
+    const int chains = static_cast<int>(std::min<size_t>(s.groups.size(), kSlotChains));
+    if (e == cudaSuccess && chains > 1) {
+        *step = "chain fork";
+        e = cudaEventRecord(s.ready, s.stream);
+        for (int k = 0; k + 1 < chains && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(s.chain[k], s.ready, 0);
+    }
     for (size_t gi = 0; e == cudaSuccess && gi < s.groups.size(); ++gi) {
         const Group& g = s.groups[gi];
         if (!g.ntiles) continue;
+        const int k = static_cast<int>(gi % static_cast<size_t>(chains));
+        const cudaStream_t st = k == 0 ? s.stream : s.chain[k - 1];
         *step = "batch kernel launch";
         gb::BatchParams p{};
         p.ngroups = 1;
@@ -166,8 +182,21 @@ cudaError_t launch_slot(scan_server* sv, Slot& s, const char** step)
         p.stages = gb::kBatchStages;
         d.slot_bytes = gb::batch_tile_blocks(g.b) * 128u * g.b;
         p.warp_bytes = p.stages * d.slot_bytes;
-        d.cta_end = 2u * static_cast<uint32_t>(sv->sms);
-        e = gb_launch_batch(false, p, gb::batch_default_warps(g.b), 2 * sv->sms, s.stream);
+        // (a small group: only as many as have a tile per warp)
+        const uint32_t w = static_cast<uint32_t>(gb::batch_default_warps(g.b));
+        const uint32_t ctas = std::min<uint32_t>(2u * static_cast<uint32_t>(sv->sms), (g.ntiles + w - 1) / w);
+        d.cta_end = ctas;
+        e = gb_launch_batch(false, p, static_cast<int>(w), static_cast<int>(ctas), st);
+    }
+    if (chains > 1) {  // joined even after a failed launch: the slot's next batch follows on its stream
+        for (int k = 0; k + 1 < chains; ++k) {
+            cudaError_t je = cudaEventRecord(s.joined[k], s.chain[k]);
+            if (je == cudaSuccess) je = cudaStreamWaitEvent(s.stream, s.joined[k], 0);
+            if (e == cudaSuccess && je != cudaSuccess) {
+                *step = "chain join";
+                e = je;
+            }
+        }
     }
     if (e == cudaSuccess) {
         // results of the n entries, then the control words (pop counters, status)
@@ -334,6 +363,11 @@ scan_status scan_server_create(scan_column* const* cols, uint32_t ncols, uint32_
         s.cap = sv->max_entries_per_batch;
         cudaError_t e = cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.ready, cudaEventDisableTiming);
+        for (int k = 0; k + 1 < kSlotChains; ++k) {
+            if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s.chain[k], cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.joined[k], cudaEventDisableTiming);
+        }
         if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&s.h_tab), s.cap * sizeof(gb::BatchCol));
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&s.d_tab), s.cap * sizeof(gb::BatchCol));
         if (e == cudaSuccess)
@@ -478,6 +512,11 @@ scan_status scan_server_destroy(scan_server* sv)
     if (sv->completer.joinable()) sv->completer.join();
     for (auto& s : sv->slots) {
         if (s.done) cudaEventDestroy(s.done);
+        if (s.ready) cudaEventDestroy(s.ready);
+        for (int k = 0; k + 1 < kSlotChains; ++k) {
+            if (s.joined[k]) cudaEventDestroy(s.joined[k]);
+            if (s.chain[k]) cudaStreamDestroy(s.chain[k]);
+        }
         if (s.stream) cudaStreamDestroy(s.stream);
         if (s.h_tab) cudaFreeHost(s.h_tab);
         if (s.h_res) cudaFreeHost(s.h_res);
