@@ -106,6 +106,14 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy()
     return p;
 }
 
+// 1 in a register the compiler cannot fold (every grid here has one z slice).
+__device__ __forceinline__ uint32_t opaque_one()
+{
+    uint32_t v;
+    asm("mov.u32 %0, %%nctaid.z;" : "=r"(v));
+    return v;
+}
+
 __device__ __forceinline__ uint32_t lanemask_lt()
 {
     uint32_t m;

@@ -208,13 +208,6 @@ __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c)
     return d;
 }
 
-__device__ __forceinline__ uint32_t opaque_one()
-{
-    uint32_t v;
-    asm("mov.u32 %0, %%nctaid.z;" : "=r"(v));
-    return v;
-}
-
 template <int B>
 __device__ __forceinline__ Lanes make_lanes(uint32_t lo, uint32_t wm1)
 {

@@ -23,12 +23,14 @@
 //                masks into row masks (lane r holds row r: values 32r..32r+31
 //                in index order), a warp scan of the row counts gives where
 //                each row's matches start, lane r writes its row's positions
-//                to the warp's shared-memory stage (padded against bank conflicts), and the warp copies the
+//                to the warp's shared-memory stage, and the warp copies the
 //                stage out with consecutive lanes on consecutive positions.
-// Branch-free visits all 32 bits of every row with a predicated store, a
-// fixed cost; branchy loops over each row's set bits only, so its cost grows
-// with the selectivity and its lanes diverge when their rows hold different
-// numbers of matches (the SIMT counterpart of a data-dependent branch).
+// Branch-free takes the same number of predicated steps in every row (as many as the
+// fullest row of a block pair has matches while rows are sparse, else 32); branchy
+// loops over each row's set bits only, so its lanes diverge when their rows hold
+// different numbers of matches (the SIMT counterpart of a data-dependent branch).
+// 2^27 values, us, branch-free before / after writing sparse blocks together: b = 16
+// 90 / 66 at sigma = 0.01, 96 / 80 at 0.1; b = 8 91 / 68 at 0.1; b = 32 125 / 109 at 0.1.
 //
 // Every wait (bulk copy, another CTA's total) is bounded by the global timer;
 // on expiry the kernel sets kErrTimeout, lets its copies in flight land and
@@ -37,6 +39,7 @@
 #include <cstdint>
 
 #include "gb_ptx.cuh"
+#include "slice.cuh"
 
 namespace gb {
 
@@ -195,6 +198,47 @@ __device__ __forceinline__ uint32_t sel_block_mask(const uint32_t* words, int la
     return pm;
 }
 
+// The widths whose count pass is bit-sliced: some 2 * B + 20..60 ALU operations a block
+// and lane against 145 of the direct one (2^27 values, sigma = 0.004 at b = 8: 66 / 51 us;
+// at b = 16, where most values match, it was 5% slower).  The column masks then hold
+// row r's bit at slice_position<B>(r).
+__host__ __device__ constexpr bool sel_sliced(int b) { return b <= 12; }
+
+// The rows below `rows` as a mask in slice order.
+template <int B>
+__device__ __forceinline__ uint32_t slice_rows(uint32_t rows)
+{
+    uint32_t m = 0u;
+#pragma unroll
+    for (int r = 0; r < 32; ++r)
+        if (static_cast<uint32_t>(r) < rows) m |= 1u << slice_position<B>(r);
+    return m;
+}
+
+template <int B>
+__device__ __forceinline__ uint32_t sel_block_mask_sliced(const uint32_t* words, int lane, const SliceKeys<B>& K,
+                                                          uint32_t limit)
+{
+    uint32_t W[B], X[B];
+#pragma unroll
+    for (int w = 0; w < B; ++w) W[w] = words[w * 32 + lane];
+    to_slices<B>(W, X, K.shift);
+    uint32_t pm = slice_match<B>(X, K);
+    if (limit < 1024u) {  // zero-padded tail block
+        const uint32_t l = static_cast<uint32_t>(lane);
+        pm &= slice_rows<B>(limit > l ? (limit - l + 31u) >> 5 : 0u);
+    }
+    return pm;
+}
+
+// The lane whose transposed mask is row `lane`'s.
+template <int B>
+__device__ __forceinline__ int slice_row_lane(int lane)
+{
+    constexpr int s = slice_segments(B), d = 32 / s;
+    return slice_odd(B) * (lane % d) % d * s + lane / d;
+}
+
 // Per-lane constants of the 32 x 32 bit transpose across the warp: stage j
 // (16, 8, 4, 2, 1) swaps the off-diagonal j x j sub-blocks.  A lane keeps the
 // bits of its own half (`keep`) and takes the partner's other half, rotated
@@ -227,28 +271,134 @@ struct Transpose {
     }
 };
 
-// Write pass over one tile.  mk[k*32 + lane] is this lane's column mask of
-// block k; the tile's matches go to pos[off ...] in index order (only those
+// Stage index of match a of a dense block (two entries of padding after every 32).
+__device__ __forceinline__ uint32_t sel_stage_at(uint32_t a) { return a + ((a >> 5) << 1); }
+
+// One match of a row to the stage, the highest bit first: entry `at` - 2 (a byte
+// address, moved down) gets code + the bit's position.  Predicated as a whole: seven
+// instructions, no branch.
+__device__ __forceinline__ void sel_step(uint32_t& m, uint32_t& at, uint32_t code)
+{
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 j, t;\n\t.reg .b16 h;\n\t"
+                 "setp.ne.u32 p, %0, 0;\n\t"
+                 "@p bfind.u32 j, %0;\n\t"
+                 "@p add.u32 %1, %1, -2;\n\t"
+                 "@p shl.b32 t, 1, j;\n\t"
+                 "@p xor.b32 %0, %0, t;\n\t"
+                 "@p add.u32 t, j, %2;\n\t"
+                 "@p cvt.u16.u32 h, t;\n\t"
+                 "@p st.shared.u16 [%1], h;\n\t}"
+                 : "+r"(m), "+r"(at)
+                 : "r"(code)
+                 : "memory");
+}
+
+// Rows of two blocks into the stage, without padding: row `lane` of block g has the
+// matches r[g], the last of which goes to entry end[g] - 1; code[g] is added to the
+// index of a match in its row.
+//   branchy    : every row loops over its set bits only (rows diverge);
+//   branch-free: all rows take as many steps as the fullest one needs, the two
+//                blocks' chains interleaved.
+template <bool BRANCHY>
+__device__ __forceinline__ void sel_scatter(const uint32_t (&r)[2], const uint32_t (&end)[2],
+                                            const uint32_t (&code)[2], uint16_t* stage)
+{
+    uint32_t m[2] = {r[0], r[1]};
+    uint32_t at[2] = {smem_u32(stage) + 2u * end[0], smem_u32(stage) + 2u * end[1]};
+    if constexpr (BRANCHY) {
+        while (m[0]) sel_step(m[0], at[0], code[0]);
+        while (m[1]) sel_step(m[1], at[1], code[1]);
+    } else {
+        const uint32_t steps =
+            __reduce_max_sync(kFull, max(static_cast<uint32_t>(__popc(m[0])), static_cast<uint32_t>(__popc(m[1]))));
+#pragma unroll 1
+        for (uint32_t i = 0; i < steps; ++i) {
+            sel_step(m[0], at[0], code[0]);
+            sel_step(m[1], at[1], code[1]);
+        }
+    }
+}
+
+// Row `lane` of one block into the padded stage, its first match at entry `at`:
+// branchy loops over the set bits, branch-free visits all 32 with a predicated store.
+template <bool BRANCHY>
+__device__ __forceinline__ void sel_scatter_block(uint32_t x, uint32_t at, uint32_t code, uint16_t* stage)
+{
+    if constexpr (BRANCHY) {
+        while (x) {
+            const uint32_t j = static_cast<uint32_t>(__ffs(static_cast<int>(x)) - 1);
+            x &= x - 1u;
+            stage[sel_stage_at(at)] = static_cast<uint16_t>(code + j);
+            ++at;
+        }
+        return;
+    }
+    // four independent chains over the row's bytes, each starting
+    // where the matches of the bytes below it end
+    uint32_t a[4] = {at, at + static_cast<uint32_t>(__popc(x & 0xffu)), at + static_cast<uint32_t>(__popc(x & 0xffffu)),
+                     at + static_cast<uint32_t>(__popc(x & 0xffffffu))};
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t bit = static_cast<uint32_t>(8 * c + j);
+            if ((x >> bit) & 1u) {  // predicated, no branch
+                stage[sel_stage_at(a[c])] = static_cast<uint16_t>(code + bit);
+                ++a[c];
+            }
+        }
+    }
+}
+
+// The stage's first `total` entries to pos[off ...], below `capacity`, each plus
+// `first`: 128 positions per step, the four stage loads before the stores.
+template <bool PADDED>
+__device__ __forceinline__ void sel_copy_out(const uint16_t* stage, uint32_t total, uint32_t first, uint32_t off,
+                                             uint32_t* pos, uint64_t capacity, int lane)
+{
+    const uint64_t room = capacity > off ? capacity - off : 0u;
+    const uint32_t lim = room < total ? static_cast<uint32_t>(room) : total;
+    for (uint32_t q0 = 0; q0 < lim; q0 += 128u) {
+        uint32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t q = q0 + 32u * u + static_cast<uint32_t>(lane);
+            v[u] = q < lim ? stage[PADDED ? sel_stage_at(q) : q] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t q = q0 + 32u * u + static_cast<uint32_t>(lane);
+            if (q < lim) pos[off + q] = first + v[u];
+        }
+    }
+}
+
+// Write pass over an iteration's blocks (at most 8).  mk[k*32 + lane] is this lane's
+// column mask of block k; the matches go to pos[off ...] in index order (only those
 // below `capacity`).  First, for all blocks at once (independent chains, so
 // their shuffle latencies overlap): a 32 x 32 bit transpose turns column masks
-// into row masks (lane r holds row r, i.e. values 32r..32r+31 in index order)
-// and a warp scan of the row counts says where each row's matches start.
-// Then per block with a match: lane r writes its row's in-block indices to
-// the warp's stage, and the warp copies the stage out with consecutive lanes
-// on consecutive positions.
-//   branch-free: every row visits its 32 bits with a predicated store;
-//   branchy    : every row loops over its set bits only (rows diverge).
-template <int TB, bool BRANCHY>
-__device__ __forceinline__ uint32_t sel_write_tile(const uint32_t* mk, uint32_t nb, uint32_t blk0, int lane,
-                                                  uint32_t off, uint32_t* pos, uint64_t capacity,
-                                                  uint16_t* stage, const Transpose& T)
+// into row masks (lane r holds row r, i.e. values 32r..32r+31 in index order;
+// `row_lane` undoes the order of bit-sliced masks) and a warp scan of the row
+// counts says where each row's matches start.  Then lane r writes its rows' indices
+// to the warp's stage, and the warp copies the stage out with consecutive lanes on
+// consecutive positions: all blocks in one go while their matches fit the stage
+// and no row has more than kSelSteps (sigma up to 1/8; block by block each paid two
+// warp syncs, a part-filled copy step and, branch-free, 32 steps), else block by block.
+constexpr uint32_t kSelSteps = 20;
+template <int TB, bool BRANCHY, bool ORDERED>
+__device__ __forceinline__ void sel_write_tile(const uint32_t* mk, uint32_t nb, uint32_t blk0, int lane,
+                                               int row_lane, uint32_t off, uint32_t* pos, uint64_t capacity,
+                                               uint16_t* stage, const Transpose& T)
 {
-    uint32_t rm[TB], incl[TB];
+    static_assert(TB <= 8, "a staged index holds 3 bits of block");
+    uint32_t rm[TB], incl[TB], most = 0u, all = 0u;
 #pragma unroll
     for (int k = 0; k < TB; ++k) {
         const uint32_t pm = static_cast<uint32_t>(k) < nb ? mk[k * 32 + lane] : 0u;
         rm[k] = T.apply(pm);
+        if constexpr (!ORDERED) rm[k] = __shfl_sync(kFull, rm[k], row_lane);
         incl[k] = static_cast<uint32_t>(__popc(rm[k]));
+        most = max(most, incl[k]);
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -259,60 +409,37 @@ __device__ __forceinline__ uint32_t sel_write_tile(const uint32_t* mk, uint32_t 
         }
     }
 #pragma unroll
+    for (int k = 0; k < TB; ++k) all += incl[k];
+    all = __shfl_sync(kFull, all, 31);
+    const uint32_t row0 = 32u * static_cast<uint32_t>(lane);
+    if (all <= 1024u && __reduce_max_sync(kFull, most) <= kSelSteps) {
+        uint32_t before = 0u;
+#pragma unroll
+        for (int k = 0; k < TB; k += 2) {
+            const bool two = k + 1 < TB;
+            const int k1 = two ? k + 1 : k;
+            const uint32_t total = __shfl_sync(kFull, incl[k], 31);
+            const uint32_t r[2] = {rm[k], two ? rm[k1] : 0u};
+            const uint32_t end[2] = {before + incl[k], before + total + incl[k1]};
+            const uint32_t code[2] = {1024u * k + row0, 1024u * k1 + row0};
+            sel_scatter<BRANCHY>(r, end, code, stage);
+            before += total + (two ? __shfl_sync(kFull, incl[k1], 31) : 0u);
+        }
+        __syncwarp();
+        sel_copy_out<false>(stage, all, blk0 * 1024u, off, pos, capacity, lane);
+        __syncwarp();
+        return;
+    }
+#pragma unroll
     for (int k = 0; k < TB; ++k) {
         const uint32_t total = __shfl_sync(kFull, incl[k], 31);
         if (total == 0u) continue;
-        uint32_t at = incl[k] - static_cast<uint32_t>(__popc(rm[k]));  // where row `lane` starts
-        const uint32_t row0 = 32u * static_cast<uint32_t>(lane);
-        if constexpr (BRANCHY) {
-            uint32_t m = rm[k];
-            while (m) {
-                const uint32_t j = static_cast<uint32_t>(__ffs(m) - 1);
-                m &= m - 1u;
-                stage[at + ((at >> 5) << 1)] = static_cast<uint16_t>(row0 + j);
-                ++at;
-            }
-        } else {
-            // four independent chains over the row's bytes, each starting
-            // where the matches of the bytes below it end
-            const uint32_t r = rm[k];
-            uint32_t a[4] = {at, at + static_cast<uint32_t>(__popc(r & 0xffu)),
-                             at + static_cast<uint32_t>(__popc(r & 0xffffu)),
-                             at + static_cast<uint32_t>(__popc(r & 0xffffffu))};
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int bit = 8 * c + j;
-                    if ((r >> bit) & 1u) {  // predicated, no branch
-                        stage[a[c] + ((a[c] >> 5) << 1)] = static_cast<uint16_t>(row0 + static_cast<uint32_t>(bit));
-                        ++a[c];
-                    }
-                }
-            }
-        }
+        sel_scatter_block<BRANCHY>(rm[k], incl[k] - static_cast<uint32_t>(__popc(rm[k])), row0, stage);
         __syncwarp();
-        const uint64_t room = capacity > off ? capacity - off : 0u;
-        const uint32_t lim = room < total ? static_cast<uint32_t>(room) : total;
-        const uint32_t first = (blk0 + static_cast<uint32_t>(k)) * 1024u;
-        // copy out 128 positions per step: the four stage loads first, then the stores
-        for (uint32_t q0 = 0; q0 < lim; q0 += 128u) {
-            uint32_t v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t q = q0 + 32u * u + static_cast<uint32_t>(lane);
-                v[u] = q < lim ? stage[q + ((q >> 5) << 1)] : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t q = q0 + 32u * u + static_cast<uint32_t>(lane);
-                if (q < lim) pos[off + q] = first + v[u];
-            }
-        }
+        sel_copy_out<true>(stage, total, (blk0 + static_cast<uint32_t>(k)) * 1024u, off, pos, capacity, lane);
         __syncwarp();
         off += total;
     }
-    return off;
 }
 
 template <int B, bool BRANCHY>
@@ -336,6 +463,11 @@ __global__ void __launch_bounds__(kSelWarps * 32, 1) k_select(const SelectParams
     const uint32_t gw = blockIdx.x * kSelWarps + warp;
     const uint32_t GW = gridDim.x * kSelWarps;
     const Transpose T(lane);
+    constexpr bool kSliced = sel_sliced(B);
+    const SliceKeys<kSliced ? B : 1> K =
+        make_slice_keys<kSliced ? B : 1>(kSliced ? p.lo : 0u, kSliced ? p.wm1 : 0u, opaque_one());
+    int row_lane = lane;
+    if constexpr (kSliced) row_lane = slice_row_lane<B>(lane);
 
     if (threadIdx.x < kSelRing) {
         cta_arrive[threadIdx.x] = 0u;
@@ -410,7 +542,9 @@ __global__ void __launch_bounds__(kSelWarps * 32, 1) k_select(const SelectParams
                 for (uint32_t k = 0; k < nb; ++k) {
                     const uint64_t blk = t * S::kTB + k;
                     const uint32_t limit = (tail && blk == nblocks - 1) ? tail : 1024u;
-                    const uint32_t pm = sel_block_mask<B>(tw + k * 32u * B, lane, p.lo, p.wm1, limit);
+                    uint32_t pm;
+                    if constexpr (kSliced) pm = sel_block_mask_sliced<B>(tw + k * 32u * B, lane, K, limit);
+                    else pm = sel_block_mask<B>(tw + k * 32u * B, lane, p.lo, p.wm1, limit);
                     mk[(m * S::kTB + k) * 32 + lane] = pm;
                     cnt += static_cast<uint32_t>(__popc(pm));
                 }
@@ -528,8 +662,8 @@ __global__ void __launch_bounds__(kSelWarps * 32, 1) k_select(const SelectParams
                 const uint32_t* mk = masks + (wi % (kSelLag + 1)) * S::kIB * 32;
                 const uint64_t left = nblocks - blk0;
                 const uint32_t nb = left < S::kIB ? static_cast<uint32_t>(left) : static_cast<uint32_t>(S::kIB);
-                sel_write_tile<S::kIB, BRANCHY>(mk, nb, static_cast<uint32_t>(blk0), lane, off, p.pos, p.capacity,
-                                                stage, T);
+                sel_write_tile<S::kIB, BRANCHY, !kSliced>(mk, nb, static_cast<uint32_t>(blk0), lane, row_lane, off,
+                                                          p.pos, p.capacity, stage, T);
             }
             base += tot;
         }

@@ -123,6 +123,14 @@ __host__ __device__ __forceinline__ void to_slices(const uint32_t (&W)[B], uint3
     }
 }
 
+// Bit position of code r (row r of a lane) in the slices.
+template <int B>
+__host__ __device__ constexpr int slice_position(int r)
+{
+    constexpr int s = slice_segments(B), d = 32 / s;
+    return slice_odd(B) * (r % d) % d * s + r / d;
+}
+
 // Block layouts.  A word of a power-of-two width holds whole codes in both, so there
 // the lane decode reads a row-major block too.
 enum Layout : int { kLayLanes = 0, kLayRow = 1 };
