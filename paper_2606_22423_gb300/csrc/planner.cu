@@ -60,7 +60,7 @@ constexpr int kTileRows = 16;
 constexpr int kThreads = 256;          // 64 units x 4 groups of 4 rows
 constexpr int kMaxOut = 16;            // strategies
 constexpr int kPadW2 = kHid + 1;       // W2's rows are read along both axes
-constexpr int kMaxParts = 128;         // CTAs of a gradient pass, each with its partial sums
+constexpr int kMaxParts = 48;          // CTAs of a gradient pass, each with its partial sums (0.9 MB in all)
 
 __host__ __device__ constexpr int param_count(int S) { return kIn * kHid + kHid + kHid * kHid + kHid + kHid * S + S; }
 
@@ -359,7 +359,7 @@ struct scan_planner {
     int step = 0;
     int cap = 0;  // rows of the output workspace (the choices' predictions)
     float* d_ws = nullptr;
-    float* d_part = nullptr;  // partial gradients, kMaxParts of them (made by the first gradient)
+    float* d_part = nullptr;  // partial gradients, kMaxParts of them
     float* d_loss = nullptr;
 
     size_t off_W(int l) const
@@ -399,7 +399,6 @@ scan_status gradients(scan_planner* pl, const float* x, const float* t, uint32_t
                       cudaStream_t st)
 {
     const int count = static_cast<int>(pl->nparams);
-    if (!pl->d_part) PL_CUDA(cudaMalloc(&pl->d_part, static_cast<size_t>(kMaxParts) * (count + 1) * sizeof(float)));
     const int tiles = static_cast<int>((rows + kTileRows - 1) / kTileRows);
     const int parts = std::min(tiles, kMaxParts);
     k_gradients<<<parts, kThreads, 0, st>>>(pl->d_params, pl->S, x, t, static_cast<int>(rows), pl->d_part);
@@ -439,7 +438,8 @@ scan_status scan_planner_create(uint32_t n_strategies, uint64_t seed, scan_plann
             h[pl->off_W(l) + i] = static_cast<float>((2.0 * u - 1.0) * lim);
         }
     }
-    cudaError_t e = cudaMalloc(&pl->d_params, 4 * pl->nparams * sizeof(float) + 16);
+    // parameters, gradients, Adam's moments, the loss; then a gradient pass's partial sums
+    cudaError_t e = cudaMalloc(&pl->d_params, (4 * pl->nparams + 4 + kMaxParts * (pl->nparams + 1)) * sizeof(float));
     if (e != cudaSuccess) {
         delete pl;
         return pcuda(e, "cudaMalloc(planner)");
@@ -448,6 +448,7 @@ scan_status scan_planner_create(uint32_t n_strategies, uint64_t seed, scan_plann
     pl->d_m = pl->d_grads + pl->nparams;
     pl->d_v = pl->d_m + pl->nparams;
     pl->d_loss = pl->d_v + pl->nparams;
+    pl->d_part = pl->d_loss + 4;
     e = cudaMemset(pl->d_params, 0, 4 * pl->nparams * sizeof(float) + 16);
     if (e == cudaSuccess) e = cudaMemcpy(pl->d_params, h.data(), pl->nparams * sizeof(float), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -465,7 +466,6 @@ scan_status scan_planner_destroy(scan_planner* pl)
     cudaDeviceSynchronize();
     if (pl->d_params) cudaFree(pl->d_params);
     if (pl->d_ws) cudaFree(pl->d_ws);
-    if (pl->d_part) cudaFree(pl->d_part);
     delete pl;
     return SCAN_OK;
 }

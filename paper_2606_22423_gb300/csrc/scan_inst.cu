@@ -110,6 +110,14 @@ cudaError_t launch_row(const ScanParams& p, const LaunchShape& sh, int grid, cud
         return launch_one<B, k_scan_full<B, BRANCHY, kLayRow>, 1>(p, sh, grid, st);
 }
 
+// Zone-skip scans: bit-sliced ones fill up their shape's warps as full scans do.
+template <int B, bool BRANCHY>
+cudaError_t launch_queue(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
+{
+    if constexpr (sliced(B, BRANCHY)) return launch_one<B, k_scan_queue<B, BRANCHY, 16>>(p, filled(B, sh), grid, st);
+    else return launch_one<B, k_scan_queue<B, BRANCHY>>(p, sh, grid, st);
+}
+
 template <int B>
 cudaError_t launch_b(int op, const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
 {
@@ -117,8 +125,8 @@ cudaError_t launch_b(int op, const ScanParams& p, const LaunchShape& sh, int gri
     switch (op) {
     case kOpFullBF: return launch_full<B, false>(p, sh, grid, st);
     case kOpFullBR: return launch_full<B, true>(p, sh, grid, st);
-    case kOpQueueBF: return launch_one<B, k_scan_queue<B, false>>(p, sh, grid, st);
-    case kOpQueueBR: return launch_one<B, k_scan_queue<B, true>>(p, sh, grid, st);
+    case kOpQueueBF: return launch_queue<B, false>(p, sh, grid, st);
+    case kOpQueueBR: return launch_queue<B, true>(p, sh, grid, st);
     case kOpZoneBuild: return launch_one<B, k_zonemap_build<B>>(p, sh, grid, st);
     case kOpRowBF: return launch_row<B, false>(p, sh, grid, st);
     case kOpRowBR: return launch_row<B, true>(p, sh, grid, st);

@@ -1098,8 +1098,9 @@ __global__ void k_zone_filter(const ScanParams p);
 // a column whose 2^20 blocks all survived spent more time in pops on the one
 // counter (~1.75 ns each) than in reading; with eight tiles per pop the warps
 // read scattered 64 KB runs and the scan ran 13% slower than the full scan.
-template <int B, bool BRANCHY>
-__global__ void __launch_bounds__(Shape<B>::kWarps * 32, 1) k_scan_queue(const ScanParams p)
+// Compiled, as the full scan, for CTAs of up to WMAX warps.
+template <int B, bool BRANCHY, int WMAX = 8>
+__global__ void __launch_bounds__(WMAX * 32, 1) k_scan_queue(const ScanParams p)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1207,7 +1208,7 @@ __global__ void __launch_bounds__(Shape<B>::kWarps * 32, 1) k_scan_queue(const S
             }
         }
     }
-    grid_finish<Shape<B>::kWarps>(p, cnt, sum, true, 0);
+    grid_finish<WMAX>(p, cnt, sum, true, 0);
 }
 
 // ----------------------------------------------------------- dispatching

@@ -79,14 +79,14 @@ gb::LaunchShape default_shape(int kind, int b)
     if (is_batch(kind))
         return gb::LaunchShape{gb::batch_default_warps(static_cast<uint32_t>(b)), gb::kBatchStages,
                                static_cast<int>(gb::batch_tile_blocks(static_cast<uint32_t>(b))), 0, 0};
-    const bool branchy = kind == kKFullBR;
-    if ((kind == kKFullBF || branchy) && gb::sliced(b, branchy)) {
-        // bit-sliced full scans (the launch fills these 8 warps up to 16): tiles of
+    const bool branchy = kind == kKFullBR || kind == kKQueueBR;
+    if (gb::sliced(b, branchy)) {
+        // bit-sliced scans (the launch fills these 8 warps up to 16): tiles of
         // 2 to 8 KB, two slots each, three at b = 5 and 6
         const int tb = b <= 2 ? 16 : (b <= 4 ? 8 : 4);
         return gb::LaunchShape{8, b == 5 || b == 6 ? 3 : 2, tb, 0, 0};
     }
-    if (branchy && gb::branchy_filled(b)) return gb::LaunchShape{8, 2, 2, 0, 0};
+    if (kind == kKFullBR && gb::branchy_filled(b)) return gb::LaunchShape{8, 2, 2, 0, 0};
     // branch-free, direct: two slots of one step instead of three of up to 8 KB,
     // except at b = 17..21 (2^28 values, three against two: 69.6 / 67.8 us at b = 13,
     // 84.2 / 79.7 at 16, 85.0 / 88.3 at 17, 107.8 / 106.9 at 22, 134.1 / 128.1 at 27,
@@ -104,7 +104,8 @@ gb::LaunchShape rule_of(int op, int b)
     if (op == gb::kOpRowBR) return default_shape(kKFullBR, b);
     if (op == gb::kOpRowBF)
         return default_shape(gb::sliced(b, false, gb::row_decode(b)) ? kKFullBR : kKFullBF, b);
-    return default_shape(kKQueueBF, b);
+    const gb::ShapeInfo si = gb::shape_of(b);
+    return gb::LaunchShape{si.warps, si.stages, si.tile_blocks, 0, 0};
 }
 
 uint32_t smem_of(int kind, int b, const gb::LaunchShape& s)
