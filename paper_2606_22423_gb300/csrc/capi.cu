@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(kFilterThreads) k_zone_filter(const ScanParams
     const uint32_t full_blocks = static_cast<uint32_t>(p.n >> 10);
     const uint32_t first = blockIdx.x * static_cast<uint32_t>(kFilterPerCta) + threadIdx.x;
     const bool agg = (p.flags & kFlagAgg) != 0u;
+    launch_dependents();  // the scan's CTAs set up meanwhile
     uint2 z[kPer];
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {

@@ -83,17 +83,33 @@ k_conj_pass(const ConjParams c, const ScanParams p)
         const uint64_t left = nblocks - t * S::kTB;
         return left < S::kTB ? static_cast<uint32_t>(left) : static_cast<uint32_t>(S::kTB);
     };
-    auto issue = [&](uint64_t t, int s) {
+    auto issue_data = [&](uint64_t t, int s) {
         const uint32_t nb = tile_blocks(t);
-        unsigned char* dst = slots + s * S::kTileBytes;
         mbar_arrive_expect_tx(&bars[s], nb * S::kBlockBytes + (kMaskIn ? nb * 128u : 0u));
-        bulk_g2s(dst, c.packed + t * S::kTB * 32u * B, nb * S::kBlockBytes, &bars[s]);
-        if constexpr (kMaskIn) bulk_g2s(dst + S::kDataBytes, c.mask + t * S::kTB * 32u, nb * 128u, &bars[s]);
+        bulk_g2s(slots + s * S::kTileBytes, c.packed + t * S::kTB * 32u * B, nb * S::kBlockBytes, &bars[s]);
     };
+    auto issue_mask = [&](uint64_t t, int s) {
+        if constexpr (kMaskIn)
+            bulk_g2s(slots + s * S::kTileBytes + S::kDataBytes, c.mask + t * S::kTB * 32u, tile_blocks(t) * 128u, &bars[s]);
+    };
+    // The next pass may start on an SM as soon as this one leaves it: it fills its
+    // slots with column data, which no pass writes, and only then waits for the end of
+    // this pass and asks for the masks.
+    launch_dependents();
     if (lane == 0) {
         for (int s = 0; s < S::kStages; ++s) {
             const uint64_t t = gw + s * GW;
-            if (t < ntiles) issue(t, s);
+            if (t < ntiles) issue_data(t, s);
+        }
+    }
+    if constexpr (kMaskIn) {
+        wait_dependency();
+        if (lane == 0) {
+            fence_proxy_async_global();
+            for (int s = 0; s < S::kStages; ++s) {
+                const uint64_t t = gw + s * GW;
+                if (t < ntiles) issue_mask(t, s);
+            }
         }
     }
     uint64_t cnt = 0, sum = 0;
@@ -137,7 +153,8 @@ k_conj_pass(const ConjParams c, const ScanParams p)
         const uint64_t tn = t + static_cast<uint64_t>(S::kStages) * GW;
         if (lane == 0 && tn < ntiles) {
             fence_proxy_async_smem();
-            issue(tn, s);
+            issue_data(tn, s);
+            issue_mask(tn, s);
         }
     }
     if (failed) {

@@ -3,6 +3,8 @@
 // global nanosecond timer so that a lost copy turns into an error status
 // instead of a hung kernel.
 #pragma once
+#include <cuda_runtime.h>
+
 #include <cstdint>
 
 namespace gb {
@@ -35,6 +37,13 @@ __device__ __forceinline__ void fence_mbar_init()
 __device__ __forceinline__ void fence_proxy_async_smem()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// Orders generic-proxy writes to global memory that this thread has come to see
+// before its later async-proxy (bulk copy) reads of them.
+__device__ __forceinline__ void fence_proxy_async_global()
+{
+    asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes)
@@ -75,6 +84,32 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
             if (mbar_try_wait(bar, parity)) return true;
         if (global_ns() - t0 > limit_ns) return false;
     }
+}
+
+// Dependent launches: lets the next kernel of the stream, if it was launched to
+// depend programmatically on this one, start before this one ends; and waits until
+// the kernel before has ended and its writes are visible.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_dependency() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Host: launches `kernel` on st, with `overlap` as a programmatic dependent of the
+// kernel before it (which must call launch_dependents, and this one wait_dependency
+// before it touches what that one writes).
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), int grid, int threads, uint32_t smem, cudaStream_t st,
+                                     bool overlap, Args&&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
 // Bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from

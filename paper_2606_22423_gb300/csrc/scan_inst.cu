@@ -54,7 +54,7 @@ inline void fit_small(const ScanParams& p, uint32_t step, LaunchShape& sh, int& 
 }
 
 template <int B, auto KERNEL, uint32_t SMALL_STEP = 0>
-cudaError_t launch_one(const ScanParams& p, LaunchShape sh, int grid, cudaStream_t st)
+cudaError_t launch_one(const ScanParams& p, LaunchShape sh, int grid, cudaStream_t st, bool overlap = false)
 {
     if (!smem_configured<KERNEL>())
         return cudaGetLastError() != cudaSuccess ? cudaGetLastError() : cudaErrorInvalidValue;
@@ -63,8 +63,9 @@ cudaError_t launch_one(const ScanParams& p, LaunchShape sh, int grid, cudaStream
     q.tile_blocks = static_cast<uint32_t>(sh.tile_blocks);
     q.stages = static_cast<uint32_t>(sh.stages);
     const uint32_t smem = pipe_smem_bytes(B, sh.warps, sh.stages, sh.tile_blocks);
-    KERNEL<<<grid, sh.warps * 32, smem, st>>>(q);
-    return cudaGetLastError();
+    // an overlapping launch's CTAs arrive as SMs come free: one per SM
+    const uint32_t least = overlap ? 116u * 1024u : 0u;
+    return launch_overlapped(KERNEL, grid, sh.warps * 32, smem > least ? smem : least, st, overlap, q);
 }
 
 // Full scans.  Bit-sliced widths take one lane per thread and one vote per two
@@ -110,12 +111,13 @@ cudaError_t launch_row(const ScanParams& p, const LaunchShape& sh, int grid, cud
         return launch_one<B, k_scan_full<B, BRANCHY, kLayRow>, 1>(p, sh, grid, st);
 }
 
-// Zone-skip scans: bit-sliced ones fill up their shape's warps as full scans do.
+// Zone-skip scans, which start while the filter before them ends (a column without a
+// whole block has no filter): bit-sliced ones fill up their shape's warps as full scans do.
 template <int B, bool BRANCHY>
 cudaError_t launch_queue(const ScanParams& p, const LaunchShape& sh, int grid, cudaStream_t st)
 {
-    if constexpr (sliced(B, BRANCHY)) return launch_one<B, k_scan_queue<B, BRANCHY, 16>>(p, filled(B, sh), grid, st);
-    else return launch_one<B, k_scan_queue<B, BRANCHY>>(p, sh, grid, st);
+    if constexpr (sliced(B, BRANCHY)) return launch_one<B, k_scan_queue<B, BRANCHY, 16>>(p, filled(B, sh), grid, st, p.n >= 1024u);
+    else return launch_one<B, k_scan_queue<B, BRANCHY>>(p, sh, grid, st, p.n >= 1024u);
 }
 
 template <int B>

@@ -1107,15 +1107,17 @@ __global__ void __launch_bounds__(WMAX * 32, 1) k_scan_queue(const ScanParams p)
     const int nwarps = static_cast<int>(blockDim.x >> 5);
     const Pipe P = pipe_of<B>(smem, p, warp, nwarps);
 
-    const uint64_t ncand = __ldcg(&p.qctl[0]);
-    const uint64_t ntiles = (ncand + P.tb - 1) / P.tb;
-    const uint64_t gw = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;
-    const uint64_t GW = static_cast<uint64_t>(gridDim.x) * nwarps;
     if (lane == 0) {
         for (uint32_t s = 0; s < P.stages; ++s) mbar_init(&P.bars[s], 1);
         fence_mbar_init();
     }
     __syncwarp();
+    const Keys<B, BRANCHY> L = make_keys<B, BRANCHY>(p.lo, p.wm1);
+    wait_dependency();  // the filter's list is complete
+    const uint64_t ncand = __ldcg(&p.qctl[0]);
+    const uint64_t ntiles = (ncand + P.tb - 1) / P.tb;
+    const uint64_t gw = static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x;
+    const uint64_t GW = static_cast<uint64_t>(gridDim.x) * nwarps;
 
     // Tile t of the candidate list: its block count and this lane's id.
     auto ids_of = [&](uint64_t t, uint32_t& id) -> uint32_t {
@@ -1158,7 +1160,6 @@ __global__ void __launch_bounds__(WMAX * 32, 1) k_scan_queue(const ScanParams p)
     uint32_t next_id = 0;
     uint32_t next_nb = tn < ntiles ? ids_of(tn, next_id) : 0u;
 
-    const Keys<B, BRANCHY> L = make_keys<B, BRANCHY>(p.lo, p.wm1);
     uint64_t cnt = 0, sum = 0;
     uint32_t it = 0, s = 0, parity = 0;
     bool failed = false;
