@@ -260,9 +260,9 @@ scan_status scan_column_status(scan_column *col, void *stream);
  * least `capacity` of them; may be NULL when capacity is 0) and the full
  * number of matches to *host_count.  Only the first min(count, capacity)
  * positions are written, so a count above capacity tells the caller how much
- * to allocate for a second call.  strategy: SCAN_BRANCHFREE (every 32-value
- * row runs the predicated store) or SCAN_BRANCHY (a warp vote per row skips
- * rows without a match); SCAN_AUTO means branch-free; the zone-skip
+ * to allocate for a second call.  strategy: SCAN_BRANCHFREE (all 32-value
+ * rows of a block pair take the same number of predicated stores) or
+ * SCAN_BRANCHY (every row loops over its matches); SCAN_AUTO means branch-free; the zone-skip
  * strategies are SCAN_EINVAL.  Both give the same positions.  One read of
  * the packed column; calls on one column must be ordered on one stream.
  * Waits for the stream; SCAN_ETIMEOUT if a bounded device wait gave up. */
@@ -305,14 +305,13 @@ typedef struct scan_batch scan_batch; /* opaque: a planned batch of column scans
 /* Plan a batch over `ncols` columns (the paper has no batched form; this
  * runs thousands of column scans as one CUDA-graph launch).  Every column's
  * blocks are cut into tiles (by default about 6 KB); columns are grouped by
- * (predicate flavour, width) and each group is served by one width-specialised
- * persistent kernel.  Groups of 16 us or more by the bandwidth law are recorded
- * as two concurrent chains of one graph: the narrow half of their widths
- * ascending, the wide half descending, so that a decode-bound and a
- * bandwidth-bound kernel share every SM (two CTAs per SM); shorter groups run
- * on six more chains, with grids in proportion to their law time.  Warps pop
- * `tiles_per_pop` consecutive tiles per
- * atomic (0 = chosen per group: at least 4, about four pops per warp).
+ * (predicate flavour, width), longest first, and the groups of four neighbouring
+ * widths whose shapes have the same warps and stages are served by one persistent
+ * kernel: its CTAs each start on one group, in proportion to the group's time by
+ * the bandwidth law, and move on when that has no tile left.  The kernels run
+ * side by side in the graph, two CTAs per SM.  Warps pop consecutive tiles by
+ * one atomic: `tiles_per_pop` of them, or with 0 a share of the group's remaining
+ * work that shrinks towards its end.
  * strategies[i] picks column i's flavour and whether it skips blocks by zone
  * map (NULL = SCAN_BRANCHFREE for all; SCAN_AUTO counts as branch-free).
  * Zone-skip columns need a built zone map.  The columns must outlive the plan.
@@ -571,8 +570,9 @@ scan_status scan_selftest_wait_timeout(uint64_t limit_ns, void *stream);
  * broken.  Nothing is written. */
 scan_status scan_selftest_select_timeout(scan_column *col, uint64_t limit_ns, void *stream);
 
-/* Number of SMs, the persistent grid size and the current shape (tuned or
- * the built-in rule) of the branch-free full scan at width b. */
+/* Number of SMs, the persistent grid size and the shape (tuned or the built-in
+ * rule, filled up as described at scan_shape) the branch-free full scan of a
+ * large column launches with at width b. */
 scan_status scan_launch_shape(uint32_t b, uint32_t *sms, uint32_t *ctas, uint32_t *warps_per_cta,
                               uint32_t *blocks_per_tile, uint32_t *stages);
 
@@ -582,15 +582,22 @@ scan_status scan_launch_shape(uint32_t b, uint32_t *sms, uint32_t *ctas, uint32_
  * single-thread decoders have no launch geometry; the shapes only change how
  * the fused scan of §3 is spread over the GPU, never its result).  One CTA per
  * SM of `warps` warps; each warp streams tiles of `tile_blocks` 1024-value
- * blocks through `stages` shared-memory slots (the zone-skip kernels pop
- * `tile_blocks` candidate blocks at a time); vote_rows = 1 makes the branchy
+ * blocks through `stages` shared-memory slots (the zone-skip kernels take
+ * `tile_blocks` candidate blocks at a time).  Bit-sliced kernels (branch-free
+ * at b <= 12, branchy at b <= 16) and the branchy full scans at b = 17..25 and
+ * b >= 28 fill a shape of at most 8 warps up: as many warps as their slots
+ * allow, in whole fours, at most twice the shape's.  A full scan of at most one
+ * tile per warp runs smaller tiles on fewer warps, on one CTA while that holds
+ * it.  vote_rows = 1 makes the branchy
  * kernel vote once per row of a thread's lanes instead of once per value, and
  * vote_rows = 2 does the same with each row written as one PTX block (tests
  * OR-ed into one predicate, one vote, one uniform branch), vote_rows = 3 with
- * two rows per block (both rows' tests and votes before either branch);
+ * two rows per block (both rows' tests and votes before either branch); bit-
+ * sliced widths vote once per two blocks whatever it says.
  * vec_lanes is how many lanes a thread reads as one vector per row: 0 (the
  * width's default: 4 for b <= 16, else 2) or 2 for full scans at b = 9..16,
- * whose smaller warp step lets 16 warps fit.  Legal shapes: full scans 1..16
+ * whose smaller warp step lets 16 warps fit (bit-sliced widths take one lane per
+ * thread whatever it says).  Legal shapes: full scans 1..16
  * warps, zone-skip scans 1..8; 1..6 stages; tile_blocks a positive multiple of
  * the warp step (vec_lanes blocks), at most 64 (full) or 32 (zone skip);
  * vote_rows only for SCAN_BRANCHY at b <= 21; warps * stages * (tile_blocks

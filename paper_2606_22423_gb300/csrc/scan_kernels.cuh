@@ -3,16 +3,18 @@
 // Paper §3: 1024-value blocks transposed over 32 lanes so that every lane
 // extracts its values with the same shifts and masks.  On the GPU a block is
 // B rows of 32 words (128*B contiguous bytes); row w holds word w of every
-// lane.  Eight threads cover one block: thread q of the group owns lanes
-// 4q..4q+3 and reads one 16-byte vector per row, so a warp works on four
-// blocks at once and every shared-memory read is conflict-free.
+// lane.  Narrow widths are decoded bit-sliced, a lane per thread (slice.cuh).  In
+// the direct decode of the others eight threads cover one block: thread q of the
+// group owns lanes 4q..4q+3 and reads one 16-byte vector per row (from b = 17, 16
+// threads of two lanes), so a warp works on four (two) blocks at once and every
+// shared-memory read is conflict-free.
 //
 // Data movement is the GB300 part: each warp runs its own pipeline of
 // kStages shared-memory slots, filled by the bulk TMA engine
 // (cp.async.bulk + mbarrier transaction counts), so ~100 KB per SM stay in
 // flight without holding registers.  The full scan walks tiles in a static
-// persistent order; the zone-skip scan pops candidate blocks from a device
-// queue (one atomic per tile).  Per-thread partials are reduced by warp
+// persistent order; the zone-skip scan walks the filter's list of surviving
+// blocks the same way.  Per-thread partials are reduced by warp
 // shuffles, then per CTA, then by the last CTA to finish (no second launch).
 #pragma once
 #include <cuda_runtime.h>

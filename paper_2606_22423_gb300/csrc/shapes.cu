@@ -9,9 +9,9 @@
 // and more warps hide its dependent chains; above it the copies bind and
 // deeper rings or larger tiles pay.  The branchy kernel adds a choice of vote
 // form (one value or one row of a thread's lanes per vote, the row as C++ or
-// as one PTX block of one or two rows).  Batched scans run two CTAs per SM
-// (one of each graph chain), so their shapes stay within half the SM's shared
-// memory.
+// as one PTX block of one or two rows).  Bit-sliced widths have one vote form and
+// one geometry, and need 16 warps: their kernels fill a shape's 8 up.  Batched scans
+// run two CTAs per SM, so their shapes stay within half the SM's shared memory.
 //
 // This unit keeps one shape per (kernel kind, b): the built-in rule until a
 // tuned shape is installed.  The tuner times every legal candidate on a
@@ -151,7 +151,7 @@ bool shape_ok(int kind, int b, const gb::LaunchShape& s, const char** why)
 // full branchy scans at b <= 21 both vote groups; illegal shapes dropped.
 // Batched scans: 4/6/8 warps, 2 or 3 stages, tiles of about 4..12 KB, only
 // shapes whose slots leave room for a second CTA on the SM (the graph runs
-// two chains of width groups side by side).
+// several launches side by side).
 std::vector<gb::LaunchShape> candidates(int kind, int b)
 {
     const bool full = kind == kKFullBF || kind == kKFullBR || is_batch(kind);
