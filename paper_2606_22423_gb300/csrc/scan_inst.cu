@@ -16,18 +16,18 @@ namespace {
 // cudaFuncSetAttribute once per (kernel, device): every instantiation may use
 // up to the whole shared-memory budget; each launch passes its own size.
 template <auto KERNEL>
-bool smem_configured()
+cudaError_t configure_smem()
 {
     static std::atomic<unsigned long long> done_mask{0ull};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
-    if (done_mask.load(std::memory_order_acquire) & bit) return true;
-    if (cudaFuncSetAttribute(reinterpret_cast<const void*>(KERNEL), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSmemMax) != cudaSuccess)
-        return false;
-    done_mask.fetch_or(bit, std::memory_order_acq_rel);
-    return true;
+    if (done_mask.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(KERNEL), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSmemMax);
+    if (e == cudaSuccess) done_mask.fetch_or(bit, std::memory_order_acq_rel);
+    return e;
 }
 
 // A full scan with at most one tile per warp of the full grid is cut finer, into
@@ -56,8 +56,7 @@ inline void fit_small(const ScanParams& p, uint32_t step, LaunchShape& sh, int& 
 template <int B, auto KERNEL, uint32_t SMALL_STEP = 0>
 cudaError_t launch_one(const ScanParams& p, LaunchShape sh, int grid, cudaStream_t st, bool overlap = false)
 {
-    if (!smem_configured<KERNEL>())
-        return cudaGetLastError() != cudaSuccess ? cudaGetLastError() : cudaErrorInvalidValue;
+    if (const cudaError_t e = configure_smem<KERNEL>(); e != cudaSuccess) return e;
     ScanParams q = p;
     if constexpr (SMALL_STEP != 0) fit_small(p, SMALL_STEP, sh, grid);
     q.tile_blocks = static_cast<uint32_t>(sh.tile_blocks);

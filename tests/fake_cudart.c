@@ -1,0 +1,117 @@
+/* A stand-in for the CUDA runtime calls of the library, preloaded by
+ * test_failed_calls.py: device memory is host memory, kernels do nothing, and a named
+ * call can be made to fail, as the runtime fails it: it returns the error and keeps it
+ * for cudaGetLastError. */
+#include <stddef.h>
+#include <stdlib.h>
+#include <string.h>
+
+typedef int err_t;
+typedef struct { unsigned x, y, z; } dim3_t;
+
+static err_t last_error;
+static char fail_name[64];
+static int fail_after = -1;
+static err_t fail_code;
+static size_t copy_bytes;
+static unsigned char symbols[1 << 16];
+
+/* The call `name` fails with `code` once, after `after` calls of it that succeed. */
+void fake_fail(const char *name, int after, int code)
+{
+    strncpy(fail_name, name, sizeof fail_name - 1);
+    fail_after = after;
+    fail_code = code;
+}
+size_t fake_copy_bytes(void) { return copy_bytes; }
+void *fake_symbols(void) { return symbols; }
+int fake_pending(void) { return fail_after >= 0; }
+
+static err_t outcome(const char *name)
+{
+    if (fail_after < 0 || strcmp(name, fail_name) != 0) return 0;
+    if (fail_after-- > 0) return 0;
+    last_error = fail_code;
+    return fail_code;
+}
+#define OUTCOME(name) do { const err_t e_ = outcome(name); if (e_) return e_; } while (0)
+
+static err_t allocate(void **p, size_t n)
+{
+    *p = aligned_alloc(256, (n + 255) / 256 * 256);
+    if (!*p) return 2;
+    memset(*p, 0, n);
+    return 0;
+}
+
+err_t cudaGetLastError(void)
+{
+    const err_t e = last_error;
+    last_error = 0;
+    return e;
+}
+err_t cudaGetDevice(int *d) { *d = 0; return 0; }
+err_t cudaDeviceGetAttribute(int *v, int attr, int dev) { (void)dev; *v = attr == 16 ? 152 : 1; return 0; }
+err_t cudaMalloc(void **p, size_t n) { OUTCOME("cudaMalloc"); return allocate(p, n); }
+err_t cudaMallocHost(void **p, size_t n) { OUTCOME("cudaMallocHost"); return allocate(p, n); }
+err_t cudaMallocAsync(void **p, size_t n, void *st) { (void)st; OUTCOME("cudaMallocAsync"); return allocate(p, n); }
+err_t cudaFree(void *p) { free(p); return 0; }
+err_t cudaFreeHost(void *p) { free(p); return 0; }
+err_t cudaFreeAsync(void *p, void *st) { (void)st; free(p); return 0; }
+err_t cudaMemset(void *p, int v, size_t n) { OUTCOME("cudaMemset"); memset(p, v, n); return 0; }
+err_t cudaMemsetAsync(void *p, int v, size_t n, void *st)
+{
+    (void)st;
+    OUTCOME("cudaMemsetAsync");
+    memset(p, v, n);
+    return 0;
+}
+err_t cudaMemcpy(void *d, const void *s, size_t n, int kind)
+{
+    (void)kind;
+    OUTCOME("cudaMemcpy");
+    copy_bytes = n;
+    memcpy(d, s, n);
+    return 0;
+}
+err_t cudaMemcpyAsync(void *d, const void *s, size_t n, int kind, void *st)
+{
+    (void)kind;
+    (void)st;
+    OUTCOME("cudaMemcpyAsync");
+    memcpy(d, s, n);
+    return 0;
+}
+err_t cudaDeviceSynchronize(void) { return 0; }
+err_t cudaStreamSynchronize(void *st) { (void)st; OUTCOME("cudaStreamSynchronize"); return 0; }
+err_t cudaStreamCreateWithFlags(void **st, unsigned f) { (void)f; *st = malloc(1); return 0; }
+err_t cudaStreamDestroy(void *st) { free(st); return 0; }
+err_t cudaFuncSetAttribute(const void *f, int attr, int v)
+{
+    (void)f;
+    (void)attr;
+    (void)v;
+    OUTCOME("cudaFuncSetAttribute");
+    return 0;
+}
+err_t cudaGetSymbolAddress(void **p, const void *sym) { (void)sym; *p = symbols; return 0; }
+/* every launch is one call named "launch" */
+err_t __cudaGetKernel(void **k, const void *f) { *k = (void *)f; return 0; }
+err_t __cudaLaunchKernel(void *k, dim3_t g, dim3_t b, void **args, size_t smem, void *st)
+{
+    (void)k; (void)g; (void)b; (void)args; (void)smem; (void)st;
+    OUTCOME("launch");
+    return 0;
+}
+err_t cudaLaunchKernelExC(const void *cfg, const void *f, void **args)
+{
+    (void)cfg; (void)f; (void)args;
+    OUTCOME("launch");
+    return 0;
+}
+err_t cudaLaunchCooperativeKernel(const void *f, dim3_t g, dim3_t b, void **args, size_t smem, void *st)
+{
+    (void)f; (void)g; (void)b; (void)args; (void)smem; (void)st;
+    OUTCOME("launch");
+    return 0;
+}
