@@ -33,7 +33,7 @@ scan_status bcuda(cudaError_t e, const char* what)
     static thread_local char buf[256];
     snprintf(buf, sizeof buf, "%s: %s", what, cudaGetErrorString(e));
     gb_set_last_error(buf);
-    return e == cudaErrorMemoryAllocation ? SCAN_ENOMEM : SCAN_ECUDA;
+    return gb_cuda_status(e);
 }
 
 #define BT_CUDA(call)                                 \
@@ -242,14 +242,11 @@ scan_status layout(scan_batch* bt)
         if (bt->d_chunks) cudaFree(bt->d_chunks);
         bt->d_chunks = nullptr;
         bt->chunk_cap = 0;
-        if (cudaMalloc(reinterpret_cast<void**>(&bt->d_chunks), chunks.size() * sizeof(uint2)) != cudaSuccess)
-            return bfail(SCAN_ENOMEM, "chunk table allocation");
+        BT_CUDA(cudaMalloc(reinterpret_cast<void**>(&bt->d_chunks), chunks.size() * sizeof(uint2)));
         bt->chunk_cap = chunks.size();
     }
-    if (!chunks.empty() &&
-        cudaMemcpy(bt->d_chunks, chunks.data(), chunks.size() * sizeof(uint2), cudaMemcpyHostToDevice) !=
-            cudaSuccess)
-        return bfail(SCAN_ECUDA, "chunk table upload");
+    if (!chunks.empty())
+        BT_CUDA(cudaMemcpy(bt->d_chunks, chunks.data(), chunks.size() * sizeof(uint2), cudaMemcpyHostToDevice));
     if (bt->graph) {
         cudaGraphExecDestroy(bt->graph);
         bt->graph = nullptr;

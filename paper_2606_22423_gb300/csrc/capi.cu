@@ -37,7 +37,7 @@ scan_status fail(scan_status s, const char* fmt, ...)
 
 scan_status cuda_fail(cudaError_t e, const char* what)
 {
-    return fail(e == cudaErrorMemoryAllocation ? SCAN_ENOMEM : SCAN_ECUDA, "%s: %s (%s)", what,
+    return fail(gb_cuda_status(e), "%s: %s (%s)", what,
                 cudaGetErrorName(e), cudaGetErrorString(e));
 }
 

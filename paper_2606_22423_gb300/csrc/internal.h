@@ -11,6 +11,15 @@
 // Sets the message scan_last_error() returns on this thread.
 void gb_set_last_error(const char* msg);
 
+// The status a failed CUDA call is reported with.  Takes the error out of
+// cudaGetLastError, where the next launch check, the library's or its caller's, would
+// find it again and report a launch that worked as failed.
+inline scan_status gb_cuda_status(cudaError_t e)
+{
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? SCAN_ENOMEM : SCAN_ECUDA;
+}
+
 // SM count and cooperative-launch support of the current device (cached per device).
 int gb_device_sms();
 bool gb_device_coop();

@@ -41,6 +41,7 @@ int g_sms[kMaxDevices] = {};
 scan_status noalloc_fail(scan_status s, const char* msg)
 {
     gb_set_last_error(msg);  // reported by scan_last_error()
+    if (s == SCAN_ECUDA) cudaGetLastError();  // reported here: not again by the next launch check
     return s;
 }
 

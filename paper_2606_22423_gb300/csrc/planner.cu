@@ -26,8 +26,7 @@
 
 #include "../../include/gbscan.h"
 #include "batch_kernels.cuh"
-
-void gb_set_last_error(const char* msg);
+#include "internal.h"
 
 namespace {
 
@@ -47,7 +46,7 @@ scan_status pcuda(cudaError_t e, const char* what)
     static thread_local char buf[256];
     snprintf(buf, sizeof buf, "%s: %s", what, cudaGetErrorString(e));
     gb_set_last_error(buf);
-    return e == cudaErrorMemoryAllocation ? SCAN_ENOMEM : SCAN_ECUDA;
+    return gb_cuda_status(e);
 }
 
 #define PL_CUDA(call)                                  \

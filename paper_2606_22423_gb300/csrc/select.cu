@@ -25,7 +25,7 @@ scan_status scuda(cudaError_t e, const char* what)
     static thread_local char buf[256];
     snprintf(buf, sizeof buf, "%s: %s", what, cudaGetErrorString(e));
     gb_set_last_error(buf);
-    return e == cudaErrorMemoryAllocation ? SCAN_ENOMEM : SCAN_ECUDA;
+    return gb_cuda_status(e);
 }
 
 #define SL_CUDA(call)                                  \

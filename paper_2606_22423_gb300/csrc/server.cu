@@ -27,10 +27,7 @@
 
 #include "../../include/gbscan.h"
 #include "batch_kernels.cuh"
-
-void gb_set_last_error(const char* msg);
-bool gb_column_view(const scan_column* c, const uint32_t** packed, uint64_t* n, uint32_t* b,
-                    uint32_t* base, const uint2** zonemap);
+#include "internal.h"
 
 namespace {
 
@@ -216,6 +213,7 @@ cudaError_t launch_slot(scan_server* sv, Slot& s, const char** step)
 
 void note_error(scan_server* sv, const char* step, cudaError_t e)
 {
+    if (e != cudaSuccess) gb_cuda_status(e);
     if (!sv->error_text[0])
         snprintf(sv->error_text, sizeof sv->error_text, "%s: %s", step,
                  e == cudaSuccess ? "device wait timed out" : cudaGetErrorString(e));
@@ -376,7 +374,7 @@ scan_status scan_server_create(scan_column* const* cols, uint32_t ncols, uint32_
             e = cudaMallocHost(reinterpret_cast<void**>(&s.h_res), (4ull * s.cap + kCtlWords) * sizeof(unsigned long long));
         if (e != cudaSuccess) {
             scan_server_destroy(sv);
-            return sfail(e == cudaErrorMemoryAllocation ? SCAN_ENOMEM : SCAN_ECUDA, "server slot allocation");
+            return sfail(gb_cuda_status(e), "server slot allocation");
         }
     }
     sv->dispatcher = std::thread(dispatcher_loop, sv);

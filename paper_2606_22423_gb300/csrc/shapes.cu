@@ -373,7 +373,8 @@ scan_status scan_autotune_column(scan_column* col, scan_pred pred, scan_strategy
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const std::vector<gb::LaunchShape> cand = candidates(kind, static_cast<int>(b));
     long long* dres = nullptr;
-    if (cudaMalloc(&dres, 32) != cudaSuccess) return shapes_fail(SCAN_ENOMEM, "cudaMalloc(result) failed");
+    if (const cudaError_t e = cudaMalloc(&dres, 32); e != cudaSuccess)
+        return shapes_fail(gb_cuda_status(e), "cudaMalloc(result) failed");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -405,7 +406,8 @@ scan_status scan_autotune_column(scan_column* col, scan_pred pred, scan_strategy
         for (uint32_t i = 0; i < k && r == SCAN_OK; ++i) r = gb_enqueue_scan(col, pred, strategy, st, dres, &empty);
         cudaEventRecord(e1, st);
         if (r != SCAN_OK) return r;
-        if (cudaEventSynchronize(e1) != cudaSuccess) return shapes_fail(SCAN_ECUDA, "a tuning launch failed");
+        if (const cudaError_t e = cudaEventSynchronize(e1); e != cudaSuccess)
+            return shapes_fail(gb_cuda_status(e), "a tuning launch failed");
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         *us = ms * 1000.f / static_cast<float>(k);

@@ -31,8 +31,11 @@ def status_of(f, *args):
         return e.status
     return gbscan.SCAN_OK
 
+memory = ctypes.create_string_buffer(1 << 16)      # kernels do nothing: only copied and set
+x = (ctypes.addressof(memory) + 255) & ~255
+
 def column(n=5000, b=8):
-    return gbscan.Column.from_packed(4096, n, b)   # an address: no kernel runs
+    return gbscan.Column.from_packed(x, n, b)
 """
 
 
@@ -63,4 +66,33 @@ def test_a_scan_whose_kernel_cannot_be_set_up_is_an_error(child):
                 fail("cudaFuncSetAttribute", code=NO_MEMORY)
                 assert status_of(c.run, 1, 5, strategy) == gbscan.SCAN_ENOMEM, (strategy, b)
                 assert status_of(c.run, 1, 5, strategy) == gbscan.SCAN_OK
+    """)
+
+
+@pytest.mark.parametrize("name", ["launch", "cudaFuncSetAttribute", "cudaMalloc", "cudaMemsetAsync"])
+def test_a_failed_call_is_not_reported_again_by_the_next_one(child, name):
+    """Launch checks read cudaGetLastError; an error that an earlier call has reported
+    must be gone from it."""
+    child(f"""
+        name = {name!r}
+        c = column(n=5000, b=8)
+        c.zonemap_build()                      # launches once, so that its kernel is set up
+        net = gbscan.Planner(4)
+        failing = {{
+            "launch": [lambda: c.run(1, 5), lambda: c.run(1, 5, "zone_bf"), lambda: c.select(1, 5),
+                       lambda: gbscan.scan_conj([c, c], [(1, 5), (1, 5)], c),
+                       lambda: gbscan.scan_run_packed_noalloc(x, 5000, 8, 0, 1, 5, x, x),
+                       lambda: net.forward(x, 16, x)],
+            "cudaFuncSetAttribute": [lambda: c.run(1, 5, "branchy"), lambda: column(b=9).select(1, 5),
+                                     lambda: gbscan.scan_conj([column(b=9)], [(1, 5)])],
+            "cudaMalloc": [lambda: column(), lambda: gbscan.Planner(4),
+                           lambda: gbscan.Batch([c], tiles_per_pop=1), lambda: c.autotune(1, 5)],
+            "cudaMemsetAsync": [lambda: c.select_async(9, 9, x, x, capacity=1),
+                                lambda: gbscan.scan_run_packed_noalloc(x, 5000, 8, 0, 1, 5, x, x)],
+        }}[name]
+        for i, f in enumerate(failing):
+            skipped = 1 if name == "launch" and i == 1 else 0    # the filter's launch, then the scan's
+            fail(name, skipped)
+            assert status_of(f) == gbscan.SCAN_ECUDA, i
+            assert rt.cudaGetLastError() == 0, i
     """)
