@@ -67,7 +67,8 @@ struct Workspace {
     unsigned int* done;
     unsigned long long* qctl;
     unsigned long long* partials;
-    static constexpr size_t kBytes = 128 + 16 * kMaxGrid;
+    static constexpr size_t kQctlBytes = 64;
+    static constexpr size_t kBytes = 64 + kQctlBytes + 16 * kMaxGrid;
 };
 
 struct DeviceInfo {
@@ -611,7 +612,13 @@ scan_status enqueue_scan(scan_column* c, scan_pred pred, scan_strategy strategy,
         }
     }
     const cudaError_t e = launch(static_cast<int>(c->b), op, p, grid, st);
-    if (e != cudaSuccess) return cuda_fail(e, "scan kernel launch");
+    if (e != cudaSuccess) {
+        // the filter's list has no reader now: left counted, the next filter would append to
+        // it, past the end of the buffer
+        if (op == gb::kOpQueueBF || op == gb::kOpQueueBR)
+            cudaMemsetAsync(c->ws.qctl, 0, Workspace::kQctlBytes, st);
+        return cuda_fail(e, "scan kernel launch");
+    }
     return SCAN_OK;
 }
 

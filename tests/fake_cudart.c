@@ -15,6 +15,8 @@ static int fail_after = -1;
 static err_t fail_code;
 static size_t copy_bytes;
 static unsigned char symbols[1 << 16];
+static struct { void *p; size_t n; } blocks[64];
+static unsigned nblocks;
 
 /* The call `name` fails with `code` once, after `after` calls of it that succeed. */
 void fake_fail(const char *name, int after, int code)
@@ -25,6 +27,13 @@ void fake_fail(const char *name, int after, int code)
 }
 size_t fake_copy_bytes(void) { return copy_bytes; }
 void *fake_symbols(void) { return symbols; }
+/* The latest of the last 64 allocations that has n bytes. */
+void *fake_block(size_t n)
+{
+    for (unsigned i = 1; i <= 64 && i <= nblocks; ++i)
+        if (blocks[(nblocks - i) % 64].n == n) return blocks[(nblocks - i) % 64].p;
+    return NULL;
+}
 int fake_pending(void) { return fail_after >= 0; }
 
 static err_t outcome(const char *name)
@@ -41,6 +50,8 @@ static err_t allocate(void **p, size_t n)
     *p = aligned_alloc(256, (n + 255) / 256 * 256);
     if (!*p) return 2;
     memset(*p, 0, n);
+    blocks[nblocks % 64].p = *p;
+    blocks[nblocks++ % 64].n = n;
     return 0;
 }
 

@@ -17,7 +17,8 @@ from paper_2606_22423_gb300 import gbscan
 
 rt = ctypes.CDLL(None)
 rt.fake_copy_bytes.restype = ctypes.c_size_t
-rt.fake_symbols.restype = ctypes.c_void_p
+rt.fake_symbols.restype = rt.fake_block.restype = ctypes.c_void_p
+rt.fake_block.argtypes = [ctypes.c_size_t]
 INVALID, NO_MEMORY = 1, 2
 
 def fail(name, after=0, code=INVALID):
@@ -95,4 +96,27 @@ def test_a_failed_call_is_not_reported_again_by_the_next_one(child, name):
             fail(name, skipped)
             assert status_of(f) == gbscan.SCAN_ECUDA, i
             assert rt.cudaGetLastError() == 0, i
+    """)
+
+
+def test_a_zone_scan_that_fails_behind_its_filter_leaves_no_candidates(child):
+    """The filter counts the surviving blocks for the scan, which resets the count; if the
+    scan is not launched, the next filter must not append to that list (it holds one entry
+    per block, so a second list would run past its end)."""
+    child("""
+        c = column(n=5000, b=8)
+        qctl = (ctypes.c_uint64 * 8).from_address(rt.fake_block(128 + 16 * 1024) + 64)   # in the column's workspace
+        c.zonemap_build()
+
+        def check(strategy):
+            qctl[0], qctl[3], qctl[4] = 4, 1024, 77                 # as the filter leaves them
+            assert status_of(c.run, 1, 5, strategy) == gbscan.SCAN_ECUDA
+            assert list(qctl) == [0] * 8, strategy
+
+        for strategy in ("zone_bf", "zone_br"):
+            fail("cudaFuncSetAttribute")
+            check(strategy)
+        for strategy in ("zone_bf", "zone_br", "zone_agg_bf", "zone_agg_br"):
+            fail("launch", 1)                                       # the filter's is the first
+            check(strategy)
     """)
