@@ -121,12 +121,14 @@ cudaError_t launch(int b, bool row, const uint32_t* v, uint64_t n, uint32_t base
 }
 
 // Error words of encoder calls in flight: each call owns one from its launch until
-// it has read it, so calls on several threads and streams don't meet.  A word is
-// zero whenever it is free.  (A word allocated per call cost 150 us: the
+// it has read it, so calls on several threads and streams don't meet.  A free word is
+// zero, or marked unknown: a call that failed may have left its error in it, and the next
+// one to take it clears it first.  (A word allocated per call cost 150 us: the
 // stream-ordered pool gives its memory back at every synchronisation.)
 constexpr int kErrWords = 64;
 __device__ unsigned int g_err_words[kErrWords];
-std::atomic<unsigned long long> g_err_used[64];  // per device, a bit per word
+std::atomic<unsigned long long> g_err_used[64];     // per device, a bit per word
+std::atomic<unsigned long long> g_err_unknown[64];  // a word's bit changes only in the hands of its owner
 
 int take_word(std::atomic<unsigned long long>& used)
 {
@@ -168,11 +170,16 @@ cudaError_t gb_encode(int b, bool rowmajor, const uint32_t* values, uint64_t n, 
     std::atomic<unsigned long long>& used = gb::g_err_used[dev & 63];
     const int i = gb::take_word(used);
     if (i >= 0) {
+        std::atomic<unsigned long long>& unknown = gb::g_err_unknown[dev & 63];
+        const unsigned long long bit = 1ull << i;
         void* words = nullptr;
         e = cudaGetSymbolAddress(&words, gb::g_err_words);
-        if (e == cudaSuccess)
-            e = gb::encode_with(static_cast<unsigned int*>(words) + i, b, rowmajor, values, n, base, out, st, error);
-        used.fetch_and(~(1ull << i), std::memory_order_release);
+        unsigned int* word = static_cast<unsigned int*>(words) + i;
+        if (e == cudaSuccess && (unknown.load() & bit)) e = cudaMemsetAsync(word, 0, sizeof *word, st);
+        if (e == cudaSuccess) e = gb::encode_with(word, b, rowmajor, values, n, base, out, st, error);
+        if (e == cudaSuccess) unknown.fetch_and(~bit);
+        else unknown.fetch_or(bit);
+        used.fetch_and(~bit, std::memory_order_release);
         return e;
     }
     // more calls in flight than words: one of this call's own

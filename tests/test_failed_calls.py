@@ -120,3 +120,22 @@ def test_a_zone_scan_that_fails_behind_its_filter_leaves_no_candidates(child):
             fail("launch", 1)                                       # the filter's is the first
             check(strategy)
     """)
+
+
+def test_an_encode_that_failed_leaves_no_error_for_the_next(child):
+    """A device encode reads its range error from one of a set of words; a call that fails
+    before it has read or cleared its word must not leave the error to a later call."""
+    child("""
+        word = ctypes.c_uint32.from_address(rt.fake_symbols())
+        encode = lambda: gbscan.scan_encode_device(x, 1000, 8, 0, x)
+        for name in ("cudaMemcpyAsync", "cudaStreamSynchronize", "cudaMemsetAsync"):   # read, wait, reset
+            word.value = 2                      # as the kernel sets it for a value out of range
+            fail(name)
+            assert status_of(encode) == gbscan.SCAN_ECUDA, name
+            assert word.value == 2
+            for _ in range(2):
+                assert status_of(encode) == gbscan.SCAN_OK, name
+        word.value = 2
+        assert status_of(encode) == gbscan.SCAN_EINVAL and word.value == 0
+        assert status_of(encode) == gbscan.SCAN_OK
+    """)
