@@ -631,9 +631,11 @@ scan_status scan_shape_set(uint32_t b, scan_strategy strategy, const scan_shape 
 scan_status scan_shape_candidates(uint32_t b, scan_strategy strategy, scan_shape *out, uint32_t capacity,
                                   uint32_t *count);
 /* Autotune the kernel of `strategy` at col's width: time every candidate on
- * this column and predicate (`reps` back-to-back scans each, on `stream`),
- * re-time the three fastest against the rule three times, interleaved, and
- * install the fastest if it beats the rule (otherwise the rule stays).
+ * this column and predicate (`reps` back-to-back scans each, on `stream`; one
+ * of those that come down to the same launch, and none that comes down to the
+ * rule's), re-time the three fastest against the rule three times, interleaved,
+ * and install the fastest if it beats the rule by more than 0.3%, about what
+ * two timings of one shape differ by (otherwise the rule stays).
  * Blocking.  Tune on a column larger than L2 (at least 2^26 values at small
  * b) so that the copies stream from HBM, with a predicate that selects
  * something; zone-skip strategies need a built zone map.  The column's

@@ -1243,6 +1243,11 @@ struct ShapeInfo {
 struct LaunchShape {
     int warps, stages, tile_blocks, vote_rows;
     int vec_lanes;  // lanes per thread and row (4 or 2; 0 = the width's default); full scans only
+    bool operator==(const LaunchShape& o) const
+    {
+        return warps == o.warps && stages == o.stages && tile_blocks == o.tile_blocks && vote_rows == o.vote_rows &&
+               vec_lanes == o.vec_lanes;
+    }
 };
 
 // Branchy full scans decoded directly whose per-value vote leaves them issue-bound

@@ -14,8 +14,8 @@
 // run two CTAs per SM, so their shapes stay within half the SM's shared memory.
 //
 // This unit keeps one shape per (kernel kind, b): the built-in rule until a
-// tuned shape is installed.  The tuner times every legal candidate on a
-// caller's column and installs the fastest; shapes can be saved to and loaded
+// tuned shape is installed.  The tuner times every launch that the legal candidates
+// come down to on a caller's column and installs the fastest; shapes can be saved to and loaded
 // from a versioned text file tied to the device they were tuned on.
 #include <cuda_runtime.h>
 
@@ -187,6 +187,39 @@ std::vector<gb::LaunchShape> candidates(int kind, int b)
     return out;
 }
 
+// What a scan with shape s launches at width b: the parts of a shape that its kernel
+// there does not look at dropped, and the warps filled up as the launch does.
+gb::LaunchShape launched(int kind, int b, gb::LaunchShape s)
+{
+    if (is_batch(kind)) return s;
+    if (s.vec_lanes == gb::default_lpt(b)) s.vec_lanes = 0;
+    if (gb::sliced(b, kind == kKFullBR || kind == kKQueueBR)) {
+        s.vote_rows = s.vec_lanes = 0;
+        return gb::filled(b, s);
+    }
+    if (kind == kKFullBR && gb::branchy_filled(b) && !s.vote_rows) {
+        const gb::LaunchShape f = gb::filled(b, s);
+        if (f.warps > 8) return f;
+    }
+    return s;
+}
+
+// The candidates a tuner has to time: one of each launch, without the rule's.
+std::vector<gb::LaunchShape> distinct(int kind, int b, const std::vector<gb::LaunchShape>& all)
+{
+    std::vector<gb::LaunchShape> seen{launched(kind, b, default_shape(kind, b))}, out;
+    for (const gb::LaunchShape& s : all) {
+        const gb::LaunchShape l = launched(kind, b, s);
+        if (std::find(seen.begin(), seen.end(), l) != seen.end()) continue;
+        seen.push_back(l);
+        out.push_back(s);
+    }
+    return out;
+}
+
+// A tuned shape is installed only for a gain above what two timings of one shape differ by.
+constexpr float kTuneGain = 0.997f;
+
 scan_status shapes_fail(scan_status s, const std::string& msg)
 {
     gb_set_last_error(msg.c_str());
@@ -240,12 +273,12 @@ gb::LaunchShape gb_shape_for(int b, int op)
     return rule_of(op, b);
 }
 
-// Candidate shapes of (op, b) for the batch tuner.
+// Candidate shapes of (op, b) for the batch tuner: without the rule's own.
 std::vector<gb::LaunchShape> gb_shape_candidates(int b, int op)
 {
     const int kind = kind_of_op(op);
     if (kind < 0 || b < 1 || b > 32) return {};
-    return candidates(kind, b);
+    return distinct(kind, b, candidates(kind, b));
 }
 
 // Install a shape for (op, b) (nullptr: the rule); false if illegal.
@@ -371,7 +404,8 @@ scan_status scan_autotune_column(scan_column* col, scan_pred pred, scan_strategy
     if (n < 1024) return shapes_fail(SCAN_EINVAL, "tune on a column of at least one whole block");
     reps = std::max<uint32_t>(1, std::min<uint32_t>(reps, 100));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const std::vector<gb::LaunchShape> cand = candidates(kind, static_cast<int>(b));
+    const std::vector<gb::LaunchShape> all = candidates(kind, static_cast<int>(b));
+    const std::vector<gb::LaunchShape> cand = distinct(kind, static_cast<int>(b), all);
     long long* dres = nullptr;
     if (const cudaError_t e = cudaMalloc(&dres, 32); e != cudaSuccess)
         return shapes_fail(gb_cuda_status(e), "cudaMalloc(result) failed");
@@ -437,11 +471,12 @@ scan_status scan_autotune_column(scan_column* col, scan_pred pred, scan_strategy
         }
         if (status == SCAN_OK) {
             def_us = acc_def / 3.f;
-            size_t bj = 0;
-            for (size_t j = 1; j < acc.size(); ++j)
-                if (acc[j] < acc[bj]) bj = j;
-            best = order[bj];
-            best_us = acc[bj] / 3.f;
+            best_us = def_us;
+            for (size_t j = 0; j < acc.size(); ++j)
+                if (acc[j] / 3.f < best_us) {
+                    best = order[j];
+                    best_us = acc[j] / 3.f;
+                }
         }
     }
     cudaEventDestroy(e0);
@@ -455,17 +490,17 @@ scan_status scan_autotune_column(scan_column* col, scan_pred pred, scan_strategy
     {
         std::lock_guard<std::mutex> lock(g_mu);
         Entry& e = g_table[kind][b];
-        const bool win = best_us < def_us;
+        const bool win = best_us < kTuneGain * def_us;
         e.tuned = win;
         e.shape = win ? cand[best] : default_shape(kind, static_cast<int>(b));
         e.best_us = win ? best_us : def_us;
         e.default_us = def_us;
         out->best = to_abi(e.shape);
+        out->best_us = e.best_us;
     }
     out->rule = to_abi(default_shape(kind, static_cast<int>(b)));
-    out->best_us = best_us < def_us ? best_us : def_us;
     out->rule_us = def_us;
-    out->candidates = static_cast<uint32_t>(cand.size());
+    out->candidates = static_cast<uint32_t>(all.size());
     return SCAN_OK;
 }
 

@@ -16,7 +16,7 @@ static err_t fail_code;
 static size_t copy_bytes;
 static unsigned char symbols[1 << 16];
 static struct { void *p; size_t n; } blocks[64];
-static unsigned nblocks;
+static unsigned nblocks, launches;
 
 /* The call `name` fails with `code` once, after `after` calls of it that succeed. */
 void fake_fail(const char *name, int after, int code)
@@ -34,6 +34,7 @@ void *fake_block(size_t n)
         if (blocks[(nblocks - i) % 64].n == n) return blocks[(nblocks - i) % 64].p;
     return NULL;
 }
+unsigned fake_launches(void) { return launches; }
 int fake_pending(void) { return fail_after >= 0; }
 
 static err_t outcome(const char *name)
@@ -44,6 +45,14 @@ static err_t outcome(const char *name)
     return fail_code;
 }
 #define OUTCOME(name) do { const err_t e_ = outcome(name); if (e_) return e_; } while (0)
+
+/* every launch is one call named "launch" */
+static err_t launch(void)
+{
+    OUTCOME("launch");
+    ++launches;
+    return 0;
+}
 
 static err_t allocate(void **p, size_t n)
 {
@@ -106,23 +115,24 @@ err_t cudaFuncSetAttribute(const void *f, int attr, int v)
     return 0;
 }
 err_t cudaGetSymbolAddress(void **p, const void *sym) { (void)sym; *p = symbols; return 0; }
-/* every launch is one call named "launch" */
+err_t cudaEventCreate(void **e) { *e = malloc(1); return 0; }
+err_t cudaEventDestroy(void *e) { free(e); return 0; }
+err_t cudaEventRecord(void *e, void *st) { (void)e; (void)st; return 0; }
+err_t cudaEventSynchronize(void *e) { (void)e; return 0; }
+err_t cudaEventElapsedTime(float *ms, void *a, void *b) { (void)a; (void)b; *ms = 1.f; return 0; }
 err_t __cudaGetKernel(void **k, const void *f) { *k = (void *)f; return 0; }
 err_t __cudaLaunchKernel(void *k, dim3_t g, dim3_t b, void **args, size_t smem, void *st)
 {
     (void)k; (void)g; (void)b; (void)args; (void)smem; (void)st;
-    OUTCOME("launch");
-    return 0;
+    return launch();
 }
 err_t cudaLaunchKernelExC(const void *cfg, const void *f, void **args)
 {
     (void)cfg; (void)f; (void)args;
-    OUTCOME("launch");
-    return 0;
+    return launch();
 }
 err_t cudaLaunchCooperativeKernel(const void *f, dim3_t g, dim3_t b, void **args, size_t smem, void *st)
 {
     (void)f; (void)g; (void)b; (void)args; (void)smem; (void)st;
-    OUTCOME("launch");
-    return 0;
+    return launch();
 }
