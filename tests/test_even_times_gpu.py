@@ -1,0 +1,47 @@
+"""Calls that do the same work in two ways take about the same time (best of many runs;
+the bounds leave room for half the difference that each once had)."""
+import pytest
+
+import synth
+from paper_2606_22423_gb300 import gbscan
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    torch.cuda.init()
+    gbscan.load()
+    gbscan.autotune_reset()
+
+
+def best_us(f, reps=20, rounds=30):
+    best = 1e9
+    for _ in range(3):
+        f()
+    for _ in range(rounds):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        for _ in range(reps):
+            f()
+        e1.record()
+        e1.synchronize()
+        best = min(best, e0.elapsed_time(e1) / reps * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("b", [5, 13, 20, 31])
+def test_a_row_major_tail_costs_no_more_than_a_lane_tail(b):
+    n = 300_001
+    v = torch.from_numpy(synth.uniform_values(synth.seed_for(71, b), n, b).view("int32")).cuda()
+    out = torch.zeros(4, dtype=torch.int64, device="cuda")
+    us = {}
+    for layout in ("lanes", "rowmajor"):
+        c = gbscan.Column.from_device(v, n, b, layout=layout)
+        us[layout] = best_us(lambda: c.run_async(1, 1 + (1 << b) // 2, out))
+        c.close()
+    assert us["rowmajor"] < 1.3 * us["lanes"], us          # was 1.6
