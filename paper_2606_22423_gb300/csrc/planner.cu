@@ -492,8 +492,21 @@ scan_status scan_planner_forward(scan_planner* pl, const float* dev_x, uint32_t 
     gb_set_last_error("");
     if (!pl || (rows && (!dev_x || !dev_y))) return pfail(SCAN_EINVAL, "null pointer");
     if (!rows) return SCAN_OK;
-    forward(pl, dev_x, static_cast<int>(rows), dev_y, static_cast<cudaStream_t>(stream));
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const size_t x_bytes = sizeof(float) * kIn * rows, y_bytes = sizeof(float) * static_cast<size_t>(pl->S) * rows;
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(dev_x), y0 = reinterpret_cast<uintptr_t>(dev_y);
+    // a tile's predictions are written while other tiles' features are still to be read: a
+    // dev_y that shares memory with dev_x gets them after the kernel
+    const bool shared = x0 < y0 + y_bytes && y0 < x0 + x_bytes;
+    float* y = dev_y;
+    if (shared) {
+        const scan_status s = ensure_ws(pl, rows);
+        if (s != SCAN_OK) return s;
+        y = pl->d_ws;
+    }
+    forward(pl, dev_x, static_cast<int>(rows), y, st);
     PL_CUDA(cudaGetLastError());
+    if (shared) PL_CUDA(cudaMemcpyAsync(dev_y, y, y_bytes, cudaMemcpyDeviceToDevice, st));
     return SCAN_OK;
 }
 
