@@ -34,9 +34,8 @@ def best_us(f, reps=20, rounds=30):
     return best
 
 
-@pytest.mark.parametrize("b", [5, 13, 20, 31])
-def test_a_row_major_tail_costs_no_more_than_a_lane_tail(b):
-    n = 300_001
+@pytest.mark.parametrize("b,n", [(5, 300_001), (13, 300_001), (20, 300_001), (31, 300_001), (16, 10_000)])
+def test_a_small_row_major_scan_costs_no_more_than_a_lane_scan(b, n):
     v = torch.from_numpy(synth.uniform_values(synth.seed_for(71, b), n, b).view("int32")).cuda()
     out = torch.zeros(4, dtype=torch.int64, device="cuda")
     us = {}
@@ -44,4 +43,4 @@ def test_a_row_major_tail_costs_no_more_than_a_lane_tail(b):
         c = gbscan.Column.from_device(v, n, b, layout=layout)
         us[layout] = best_us(lambda: c.run_async(1, 1 + (1 << b) // 2, out))
         c.close()
-    assert us["rowmajor"] < 1.3 * us["lanes"], us          # was 1.6
+    assert us["rowmajor"] < 1.3 * us["lanes"], us          # was 1.45 to 1.6
