@@ -72,8 +72,17 @@ constexpr double kShortestUs = 5.0;
 // about kColumnCost: pops shrink towards the end, where the short columns are.
 // (Equal pops of a quarter of a warp's share: 11% slower on the same 1024 columns;
 // a least pop of 3 tiles instead of one: 4% slower.)
+// Not below what the group's counter can hand out: it serves a pop in about kPopUs, and
+// with all warps of the GPU on one group single tiles are decoded as fast as that.  Where
+// no zone map is asked the least pop keeps the counter busy half the time at most; where
+// one is, the tiles left cluster in few pops, and a longer one costs more than the wait.
+// us per replay, least pop of one tile / of this rule / equal pops of at least 4: 4 columns
+// of 2^24 values at b = 20 46 / 36 / 37, at b = 8 35.5 / 26 / 26.5, 16 of 2^24 at b = 20
+// 86 / 80 / 81; one sorted column of 2^24, zone skipping at 0.3, b = 20 21.0 / 19.4 / 21.9
+// (25.6 with the counter idle half the time).
 constexpr double kPopPart = 2.0;
 constexpr double kColumnCost = 1.5;
+constexpr double kPopUs = 1.75e-3;
 
 }  // namespace
 
@@ -92,6 +101,7 @@ struct scan_batch {
         uint32_t chunk_off;  // offset of this group's pops in the chunk table
         gb::LaunchShape shape;  // warps, stages and tile blocks of this width group
         double bytes;           // packed bytes of its columns
+        bool zone;              // a column of it skips by zone map
     };
     std::vector<Group> groups;
     struct Launch {  // groups of one flavour, range of widths, warps and stages
@@ -151,7 +161,7 @@ scan_status layout(scan_batch* bt)
         const int k = bt->kernel_of[i];
         if (bt->groups.empty() || bt->groups.back().kernel != k ||
             bt->groups.back().b != static_cast<int>(width[i])) {
-            scan_batch::Group g{k, static_cast<int>(width[i]), j, 0, 0, 1, 1, 0, {}, 0.0};
+            scan_batch::Group g{k, static_cast<int>(width[i]), j, 0, 0, 1, 1, 0, {}, 0.0, false};
             g.shape = gb_shape_for(g.b, k == 1 ? gb::kOpBatchBR : gb::kOpBatchBF);
             bt->groups.push_back(g);
             group_tiles = 0;
@@ -175,6 +185,7 @@ scan_status layout(scan_batch* bt)
         if (group_tiles + t > 0xffffffffull) return bfail(SCAN_EINVAL, "too many tiles in one batch");
         group_tiles += static_cast<uint32_t>(t);
         bt->groups.back().bytes += static_cast<double>(nblocks) * 128.0 * b;
+        bt->groups.back().zone |= bt->zone[i] != 0u;
         bt->groups.back().count += 1;
         bt->groups.back().ntiles = group_tiles;
         bt->slot_of[i] = j;
@@ -210,6 +221,8 @@ scan_status layout(scan_batch* bt)
             at->grid += g.ctas;
         }
         const double warps = static_cast<double>(g.ctas) * static_cast<double>(gw);
+        const double least = std::ceil((g.zone ? 1.0 : 2.0) * kPopUs * g.ctas / static_cast<double>(cap) * g.ntiles /
+                                       law_us(g.bytes, g.b));
         double left = static_cast<double>(g.ntiles) + kColumnCost * g.count;
         g.chunk_off = static_cast<uint32_t>(chunks.size());
         uint32_t col = g.first, t = 0;
@@ -220,7 +233,7 @@ scan_status layout(scan_batch* bt)
                 t = std::min(g.ntiles, t + bt->tiles_per_pop);
                 continue;
             }
-            const double want = std::max(1.0, left / (kPopPart * warps));
+            const double want = std::max(least, left / (kPopPart * warps));
             double got = 0.0;
             uint32_t c = col;
             while (t < g.ntiles && got < want) {
