@@ -83,6 +83,12 @@ constexpr double kShortestUs = 5.0;
 constexpr double kPopPart = 2.0;
 constexpr double kColumnCost = 1.5;
 constexpr double kPopUs = 1.75e-3;
+// The graph's descriptor copy and its reset of the results run side by side only for
+// larger tables; up to this size the copy is short and one after the other starts the
+// kernels sooner.  us per replay one after the other / side by side, columns of 5000 values:
+// 1 column at b = 8 14.1 / 16.3, 64 at b = 20 19.7 / 20.3, 256 of four widths 30.9 / 31.5,
+// 384 at b = 8 29.1 / 26.3, 384 of four widths 32.2 / 29.5, 1024 of all widths 48.0 / 43.2.
+constexpr size_t kSideBySideBytes = 24 * 1024;
 
 }  // namespace
 
@@ -638,8 +644,8 @@ scan_status scan_batch_exec(scan_batch* bt, const scan_pred* preds, void* stream
     const size_t res_words = 4ull * std::max<uint32_t>(1, bt->ncols) + kCtlWords;
     unsigned long long* ctl = bt->d_results + 4ull * std::max<uint32_t>(1, bt->ncols);
     if (!bt->graph) {
-        // {copy descriptors, reset results and counters} -> the launches, side by
-        // side: captured on one stream whose dependencies are set by hand
+        // {copy descriptors, reset results and counters, see kSideBySideBytes} -> the
+        // launches, side by side: captured on one stream whose dependencies are set by hand
         cudaStream_t cs = bt->capture_stream;
         BT_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
         std::vector<cudaGraphNode_t> roots, ends;
@@ -657,9 +663,11 @@ scan_status scan_batch_exec(scan_batch* bt, const scan_pred* preds, void* stream
                                                          cudaStreamSetCaptureDependencies);
         };
         ce = cudaMemcpyAsync(bt->d_table, bt->h_table, table_bytes, cudaMemcpyHostToDevice, cs);
-        note(roots);
-        std::vector<cudaGraphNode_t> none;
-        after(none);
+        if (table_bytes > kSideBySideBytes) {
+            note(roots);
+            std::vector<cudaGraphNode_t> none;
+            after(none);
+        }
         if (ce == cudaSuccess) ce = cudaMemsetAsync(bt->d_results, 0, res_words * sizeof(unsigned long long), cs);
         note(roots);
         for (const auto& l : bt->launches) {

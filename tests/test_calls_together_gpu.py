@@ -93,3 +93,24 @@ def test_scans_enqueued_without_a_wait_are_exact():
     for c in cols:
         c.status()
         c.close()
+
+
+@pytest.mark.parametrize("ncols", [3, 340, 342, 700])
+def test_batch_replays_with_new_predicates_are_exact(ncols):
+    """Small and large descriptor tables (copied before the reset of the results, or beside
+    it): replays without a wait between, each with predicates of its own."""
+    widths = [4 + i % 9 for i in range(ncols)]
+    vals = [synth.uniform_values(synth.seed_for(63, i), 900 + 37 * (i % 50), b) for i, b in enumerate(widths)]
+    cols = [gbscan.Column.from_host(v, b) for v, b in zip(vals, widths)]
+    bt = gbscan.Batch(cols)
+    out = torch.zeros((4, ncols, 4), dtype=torch.int64, device="cuda")
+    preds = [[synth.pick_range(synth.seed_for(63, i, k), b, 0.2 * (k + 1)) for i, b in enumerate(widths)] for k in range(4)]
+    for k in range(4):
+        bt.run(preds[k], dev_out=out[k], host=False)
+    got = out.cpu().numpy()
+    for k in range(4):
+        for i, v in enumerate(vals):
+            assert (int(got[k, i, 0]), int(got[k, i, 1])) == tuple(oracle.scan_values(v, *preds[k][i])), (k, i)
+    bt.close()
+    for c in cols:
+        c.close()
