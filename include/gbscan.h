@@ -310,8 +310,8 @@ typedef struct scan_batch scan_batch; /* opaque: a planned batch of column scans
  * kernel: its CTAs each start on one group, in proportion to the group's time by
  * the bandwidth law, and move on when that has no tile left.  The kernels run
  * side by side in the graph, two CTAs per SM.  Warps pop consecutive tiles by
- * one atomic: `tiles_per_pop` of them, or with 0 a share of the group's remaining
- * work that shrinks towards its end.
+ * one atomic: `tiles_per_pop` of them (1024 at most), or with 0 a share of the
+ * group's remaining work that shrinks towards its end.
  * strategies[i] picks column i's flavour and whether it skips blocks by zone
  * map (NULL = SCAN_BRANCHFREE for all; SCAN_AUTO counts as branch-free).
  * Zone-skip columns need a built zone map.  The columns must outlive the plan.

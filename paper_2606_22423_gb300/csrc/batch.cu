@@ -83,6 +83,8 @@ constexpr double kShortestUs = 5.0;
 constexpr double kPopPart = 2.0;
 constexpr double kColumnCost = 1.5;
 constexpr double kPopUs = 1.75e-3;
+// The most of a caller's tiles_per_pop: a pop is one warp's work.
+constexpr uint32_t kMostTilesPerPop = 1024;
 // The graph's descriptor copy and its reset of the results run side by side only for
 // larger tables; up to this size the copy is short and one after the other starts the
 // kernels sooner.  us per replay one after the other / side by side, columns of 5000 values:
@@ -236,7 +238,7 @@ scan_status layout(scan_batch* bt)
             while (col + 1 < g.first + g.count && bt->h_table[col + 1].tile_begin <= t) ++col;
             chunks.push_back(make_uint2(t, col - g.first));
             if (bt->tiles_per_pop) {
-                t = std::min(g.ntiles, t + bt->tiles_per_pop);
+                t += std::min({g.ntiles - t, bt->tiles_per_pop, kMostTilesPerPop});
                 continue;
             }
             const double want = std::max(least, left / (kPopPart * warps));

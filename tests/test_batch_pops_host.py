@@ -28,3 +28,14 @@ def test_pops_of_one_width_keep_within_their_counter(child, b):  # noqa: F811
                     assert pops * 1.75e-3 <= share * us + 1.0 or pops <= 2 * warps, (ncols, n, strategy, pops, us)
                     bt.close()
     """)
+
+
+def test_pops_of_a_given_size_stay_within_a_warps_work(child):  # noqa: F811
+    child("""
+        b, n = 8, 60_000 * 1024
+        tiles = -(-60_000 // gbscan.batch_shape_get(b)["tile_blocks"])
+        for per_pop in (1, 7, 1000, 1024, 1025, 1 << 20, (1 << 32) - 1):
+            bt = gbscan.Batch([column(n=n, b=b)], tiles_per_pop=per_pop)
+            assert rt.fake_copy_bytes() // 8 - 1 == -(-tiles // min(per_pop, 1024)), per_pop
+            bt.close()
+    """)
