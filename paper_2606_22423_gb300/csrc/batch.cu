@@ -85,11 +85,12 @@ constexpr double kColumnCost = 1.5;
 constexpr double kPopUs = 1.75e-3;
 // The most of a caller's tiles_per_pop: a pop is one warp's work.
 constexpr uint32_t kMostTilesPerPop = 1024;
-// The graph's descriptor copy and its reset of the results run side by side only for
-// larger tables; up to this size the copy is short and one after the other starts the
-// kernels sooner.  us per replay one after the other / side by side, columns of 5000 values:
-// 1 column at b = 8 14.1 / 16.3, 64 at b = 20 19.7 / 20.3, 256 of four widths 30.9 / 31.5,
-// 384 at b = 8 29.1 / 26.3, 384 of four widths 32.2 / 29.5, 1024 of all widths 48.0 / 43.2.
+// The graph's descriptor copy and its reset of the results run side by side, but one after
+// the other before a single launch with a table up to this size: the copy is short then, and
+// a kernel behind one node starts sooner.  us per replay one after the other / side by side,
+// columns of 5000 values: 1 column at b = 8 14.1 / 16.3, 64 at b = 20 19.7 / 20.3, 256 at
+// b = 5..8 30.9 / 31.5, 384 at b = 8 29.1 / 26.3.  Several launches start in another order
+// behind one node: 256 columns of 2^30 values of all widths 424 / 389, 192 of 2^28 130 / 126.
 constexpr size_t kSideBySideBytes = 24 * 1024;
 
 }  // namespace
@@ -665,7 +666,7 @@ scan_status scan_batch_exec(scan_batch* bt, const scan_pred* preds, void* stream
                                                          cudaStreamSetCaptureDependencies);
         };
         ce = cudaMemcpyAsync(bt->d_table, bt->h_table, table_bytes, cudaMemcpyHostToDevice, cs);
-        if (table_bytes > kSideBySideBytes) {
+        if (bt->launches.size() != 1 || table_bytes > kSideBySideBytes) {
             note(roots);
             std::vector<cudaGraphNode_t> none;
             after(none);
