@@ -198,11 +198,14 @@ __device__ __forceinline__ uint32_t sel_block_mask(const uint32_t* words, int la
     return pm;
 }
 
-// The widths whose count pass is bit-sliced: some 2 * B + 20..60 ALU operations a block
-// and lane against 145 of the direct one (2^27 values, sigma = 0.004 at b = 8: 66 / 51 us;
-// at b = 16, where most values match, it was 5% slower).  The column masks then hold
-// row r's bit at slice_position<B>(r).
-__host__ __device__ constexpr bool sel_sliced(int b) { return b <= 12; }
+// The widths whose count pass is bit-sliced: fewer ALU operations a block and lane than the
+// 145 of the direct one (2^27 values, sigma = 0.004 at b = 8: 66 / 51 us).  Time of the direct
+// form over the sliced one's, both flavours and seven selectivities: with 2^26 values 1.05 at
+// b = 9, 1.03 at 10, 1.04 at 11, 1.00 at 12; with 10^6 to 1.6 10^7 1.03, 1.03, 1.02 and 0.975;
+// a column of one block is scanned faster direct (0.90 to 0.95 at b = 9..11), its keys made for
+// it alone.  At b = 16, where most values match, the sliced form was 5% slower.  The column
+// masks then hold row r's bit at slice_position<B>(r).
+__host__ __device__ constexpr bool sel_sliced(int b) { return b <= 11; }
 
 // The rows below `rows` as a mask in slice order.
 template <int B>

@@ -96,10 +96,12 @@ def test_scans_enqueued_without_a_wait_are_exact():
 
 
 @pytest.mark.parametrize("ncols", [3, 340, 342, 700])
-def test_batch_replays_with_new_predicates_are_exact(ncols):
-    """Small and large descriptor tables (copied before the reset of the results, or beside
-    it): replays without a wait between, each with predicates of its own."""
-    widths = [4 + i % 9 for i in range(ncols)]
+@pytest.mark.parametrize("spread", [4, 9])
+def test_batch_replays_with_new_predicates_are_exact(ncols, spread):
+    """One launch and several, small and large descriptor tables (copied before the reset
+    of the results, or beside it): replays without a wait between, each with predicates of
+    its own."""
+    widths = [5 + i % spread for i in range(ncols)]
     vals = [synth.uniform_values(synth.seed_for(63, i), 900 + 37 * (i % 50), b) for i, b in enumerate(widths)]
     cols = [gbscan.Column.from_host(v, b) for v, b in zip(vals, widths)]
     bt = gbscan.Batch(cols)
