@@ -114,7 +114,7 @@ struct scan_batch {
     };
     std::vector<Group> groups;
     struct Launch {  // groups of one flavour, range of widths, warps and stages
-        int kernel, warps, stages, grid;
+        int kernel, warps, stages;
         std::vector<size_t> groups;
     };
     std::vector<Launch> launches;
@@ -223,11 +223,10 @@ scan_status layout(scan_batch* bt)
                     at = &l;
             }
             if (!at) {
-                bt->launches.push_back({g.kernel, g.shape.warps, g.shape.stages, 0, {}});
+                bt->launches.push_back({g.kernel, g.shape.warps, g.shape.stages, {}});
                 at = &bt->launches.back();
             }
             at->groups.push_back(gi);
-            at->grid += g.ctas;
         }
         const double warps = static_cast<double>(g.ctas) * static_cast<double>(gw);
         const double least = std::ceil((g.zone ? 1.0 : 2.0) * kPopUs * g.ctas / static_cast<double>(cap) * g.ntiles /

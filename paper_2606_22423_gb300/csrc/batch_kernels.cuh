@@ -432,5 +432,3 @@ inline cudaError_t gb_launch_batch(bool branchy, const gb::BatchParams& p, int w
     }
 #undef GB_RANGE
 }
-
-

@@ -303,15 +303,6 @@ __device__ __forceinline__ void acc1_fma(uint32_t& c, uint32_t& a, uint32_t ui, 
         : "+r"(c), "+r"(a) : "r"(ui), "r"(L.negloi), "r"(L.wm1), "r"(L.one));
 }
 
-// packed accumulator: a += v + add when lo <= v < hi (compares on the ALU)
-__device__ __forceinline__ void acc0_imad(uint32_t& a, uint32_t ui, const Lanes& L)
-{
-    asm("{\n\t.reg .pred p;\n\t"
-        "setp.ge.u32 p, %1, %2;\n\t"
-        "setp.lt.and.u32 p, %1, %3, p;\n\t"
-        "@p mad.lo.u32 %0, %1, %4, %0;\n\t}"
-        : "+r"(a) : "r"(ui), "r"(L.loi), "r"(L.hii), "r"(L.one));
-}
 // subtract on the FMA pipe, compare and add on the ALU (a top-of-word field,
 // whose extraction was already an IMAD)
 __device__ __forceinline__ void acc0_fsub(uint32_t& a, uint32_t ui, const Lanes& L)
@@ -321,14 +312,6 @@ __device__ __forceinline__ void acc0_fsub(uint32_t& a, uint32_t ui, const Lanes&
         "setp.le.u32 p, t, %3;\n\t"
         "@p add.u32 %0, %0, %1;\n\t}"
         : "+r"(a) : "r"(ui), "r"(L.negloi), "r"(L.wm1), "r"(L.one));
-}
-__device__ __forceinline__ void acc0_alu(uint32_t& a, uint32_t ui, const Lanes& L)
-{
-    asm("{\n\t.reg .pred p;\n\t"
-        "setp.ge.u32 p, %1, %2;\n\t"
-        "setp.lt.and.u32 p, %1, %3, p;\n\t"
-        "@p add.u32 %0, %0, %1;\n\t}"
-        : "+r"(a) : "r"(ui), "r"(L.loi), "r"(L.hii));
 }
 // 32-bit sum + count
 __device__ __forceinline__ void acc1_imad(uint32_t& c, uint32_t& a, uint32_t ui, const Lanes& L)
@@ -1229,13 +1212,15 @@ struct ShapeInfo {
 
 // A runtime launch shape: CTAs of `warps` warps (one per SM for single-column
 // scans, two for batched ones), each warp with `stages` slots of `tile_blocks`
-// blocks (the zone-skip kernels take that many candidates per tile); vote_rows
-// picks the branchy vote form (0 per value, 1 per row, 2 and 3 the PTX row
-// blocks; full branchy scans at b <= 21 only); vec_lanes = 2 the 2-lane
-// geometry (full scans at b = 9..16, compiled with the 16-warp bound).  Full
-// scans take 8..16 warps (above 8, and for vote forms 2 and 3, the
-// 16-warp-bound instantiation, <= 128 registers per thread); every other
-// single-column kernel 1..8.
+// blocks (the zone-skip kernels take that many candidates per tile).  Two parts are
+// for direct decoders only, bit-sliced kernels look at neither: vote_rows picks the
+// vote form of full branchy scans (0 per value, 1 per row, 2 and 3 the PTX row
+// blocks; accepted to b = 21, at work at 17..21), and vec_lanes = 2 the 2-lane
+// geometry of full branch-free scans (accepted at b = 9..16, at work at 13..16,
+// compiled with the 16-warp bound).  Accepted are 1..16 warps for full and batched
+// scans (above 8, and for vote forms 2 and 3, the 16-warp-bound instantiation, <= 128
+// registers per thread) and 1..8 for zone-skip scans; kernels with the 16-warp bound
+// of either kind, and row-major ones, fill a shape of 8 up (filled()).
 struct LaunchShape {
     int warps, stages, tile_blocks, vote_rows;
     int vec_lanes;  // lanes per thread and row (4 or 2; 0 = the width's default); full scans only

@@ -30,7 +30,7 @@
 // loops over each row's set bits only, so its lanes diverge when their rows hold
 // different numbers of matches (the SIMT counterpart of a data-dependent branch).
 // 2^27 values, us, branch-free before / after writing sparse blocks together: b = 16
-// 90 / 66 at sigma = 0.01, 96 / 80 at 0.1; b = 8 91 / 68 at 0.1; b = 32 125 / 109 at 0.1.
+// 90 / 66 at sigma = 0.01, 96 / 78 at 0.1; b = 8 91 / 68 at 0.1; b = 32 125 / 109 at 0.1.
 //
 // Every wait (bulk copy, another CTA's total) is bounded by the global timer;
 // on expiry the kernel sets kErrTimeout, lets its copies in flight land and

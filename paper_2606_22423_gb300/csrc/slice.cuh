@@ -15,9 +15,9 @@
 //   digit j of every code into one word, and a rotation by j digits brings code c
 //   to position m*c mod D for every j.  k butterfly stages over the 2^k segments
 //   then split the digits into bits (a shift and a select per word and stage).
-// Per 32 codes that is 8 ALU operations at B = 3, 19 at 5, 22 at 6, 27 at 7, 24 at 8,
-// 44 at 9, 48 at 10, 56 at 12 and 68 at 14, with the shifts (2 per pair of words
-// and stage) as multiplications on the FMA pipe.
+// Per 32 codes that is 8 ALU operations at B = 3, 19 at 5, 25 at 6, 27 at 7, 36 at 8,
+// 44 at 9, 53 at 10, 68 at 12 and 75 at 14, with the left one of the two shifts per pair
+// of words and butterfly stage as a multiplication on the FMA pipe beside them.
 //
 // The range test then runs on all 32 codes at once: u >= lo and u > hi are
 // carry chains of B majorities (one LOP3 each) from the lowest bit up, the count
@@ -56,9 +56,9 @@ struct SliceShifts {
     uint32_t mul[5];  // 2^(1 << e)
 };
 
-// (a & mask) | (b & ~mask).  On the device one LOP3, spelled out: from the
-// expression the compiler made two, with the mask and its complement as separate
-// immediates.
+// (a & mask) | (b & ~mask).  On the device spelled out as one LOP3: written as the
+// expression the scans took up to 1.28 times as long (2^28 values, us, expression / spelled
+// out: 34.8 / 30.8 at b = 5, 51.3 / 43.8 at 8, 77.9 / 63.7 at 12, branchy 101.3 / 81.9 at 16).
 #ifdef __CUDA_ARCH__
 __device__ __forceinline__ uint32_t bit_select(uint32_t a, uint32_t b, uint32_t mask)
 {
@@ -170,14 +170,8 @@ __device__ __forceinline__ SliceKeys<B> make_slice_keys(uint32_t lo, uint32_t wm
         K.lo[i] = ((lo >> i) & 1u) - 1u;
         K.hi[i] = ((last >> i) & 1u) - 1u;
     }
-    // kept in registers: recomputed in the loop they cost an ALU operation each
 #pragma unroll
-    for (int i = 0; i < B; ++i) asm volatile("" : "+r"(K.lo[i]), "+r"(K.hi[i]));
-#pragma unroll
-    for (int e = 0; e < 5; ++e) {
-        K.shift.mul[e] = one << (1 << e);
-        asm volatile("" : "+r"(K.shift.mul[e]));
-    }
+    for (int e = 0; e < 5; ++e) K.shift.mul[e] = one << (1 << e);
     return K;
 }
 
