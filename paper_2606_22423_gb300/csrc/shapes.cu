@@ -82,11 +82,11 @@ gb::LaunchShape default_shape(int kind, int b)
     const bool branchy = kind == kKFullBR || kind == kKQueueBR;
     if (gb::sliced(b, branchy)) {
         // bit-sliced scans (the launch fills these 8 warps up to 16): tiles of 2 to 8 KB, two
-        // slots each (2^28 values, two / three slots, us: 26.3 / 27.7 at b = 4, 30.9 / 30.8
-        // at 5, 35.0 / 35.1 at 6, 39.2 / 41.5 at 7, 43.6 / 45.8 at 8, 63.8 / 66.4 at 12;
-        // branchy 81.6 / 94.0 at 16)
+        // slots each, but three at b = 5 (2^28 values, two / three slots, us: 26.3 / 27.7 at
+        // b = 4, 30.92 / 30.75 at 5, 35.0 / 35.1 at 6, 39.2 / 41.5 at 7, 43.6 / 45.8 at 8,
+        // 63.8 / 66.4 at 12; branchy 81.6 / 94.0 at 16)
         const int tb = b <= 2 ? 16 : (b <= 4 ? 8 : 4);
-        return gb::LaunchShape{8, 2, tb, 0, 0};
+        return gb::LaunchShape{8, b == 5 ? 3 : 2, tb, 0, 0};
     }
     if (kind == kKFullBR && gb::branchy_filled(b)) return gb::LaunchShape{8, 2, 2, 0, 0};
     // branch-free, direct: two slots of one step instead of three of up to 8 KB,
