@@ -358,9 +358,9 @@ __device__ __forceinline__ bool batch_group(const BatchGroup& P, unsigned long l
 // A kernel serves a range of four widths.  Every CTA starts on one of the launch's
 // width groups (its share of the CTAs follows its law time) and its warps go on to
 // the next when that has no tile left, so that a group finished early -- zone maps
-// skipped most of it -- leaves no SM idle, and a batch of all 32 widths takes 8
-// launches side by side instead of 32 in chains (each of those cost some 12 us of
-// ramp and drain).  Compiled for CTAs of up to 16 warps, which caps it at 128
+// skipped most of it -- leaves no SM idle, and a batch of all 32 widths takes 12
+// launches side by side (widths of one range part where their shapes have fewer warps)
+// instead of 32 in chains (each of those cost some 12 us of ramp and drain).  Compiled for CTAs of up to 16 warps, which caps it at 128
 // registers a thread: two 8-warp CTAs then fit one SM.
 template <bool BRANCHY, int LO>
 __global__ void __launch_bounds__(512, 1) k_scan_batch(const __grid_constant__ BatchParams P)
