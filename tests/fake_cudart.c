@@ -16,7 +16,7 @@ static err_t fail_code;
 static size_t copy_bytes;
 static unsigned char symbols[1 << 16];
 static struct { void *p; size_t n; } blocks[64];
-static unsigned nblocks, launches;
+static unsigned nblocks, launches, last_grid, last_block;
 
 /* The call `name` fails with `code` once, after `after` calls of it that succeed. */
 void fake_fail(const char *name, int after, int code)
@@ -35,6 +35,9 @@ void *fake_block(size_t n)
     return NULL;
 }
 unsigned fake_launches(void) { return launches; }
+/* Grid and block size of the last launch by cudaLaunchKernelExC. */
+unsigned fake_grid(void) { return last_grid; }
+unsigned fake_block_size(void) { return last_block; }
 int fake_pending(void) { return fail_after >= 0; }
 
 static err_t outcome(const char *name)
@@ -128,7 +131,9 @@ err_t __cudaLaunchKernel(void *k, dim3_t g, dim3_t b, void **args, size_t smem, 
 }
 err_t cudaLaunchKernelExC(const void *cfg, const void *f, void **args)
 {
-    (void)cfg; (void)f; (void)args;
+    (void)f; (void)args;
+    last_grid = ((const dim3_t *)cfg)[0].x;   /* the configuration begins with the two sizes */
+    last_block = ((const dim3_t *)cfg)[1].x;
     return launch();
 }
 err_t cudaLaunchCooperativeKernel(const void *f, dim3_t g, dim3_t b, void **args, size_t smem, void *st)

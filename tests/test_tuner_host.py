@@ -1,6 +1,7 @@
-"""What the autotuner times, on CPU (the runtime's calls replaced, kernels do nothing):
-several candidate shapes run the same kernel in the same way at the bit-sliced widths, and
-each launch is timed once, the rule's only as the rule."""
+"""Launches as the host makes them, on CPU (the runtime's calls replaced, kernels do nothing).
+The autotuner: several candidate shapes run the same kernel in the same way at the
+bit-sliced widths, and each launch is timed once, the rule's only as the rule.  Small
+columns: cut into tiles of one step of the decode, on one CTA while that holds them."""
 import pytest
 
 from tests.test_failed_calls import child  # noqa: F401
@@ -36,4 +37,25 @@ def test_every_launch_is_timed_once(child, kind):  # noqa: F811
             assert rt.fake_launches() - before == scans * (2 if kind.startswith("zone") else 1), b
             assert r["best"] == rule and r["best_us"] == r["rule_us"], b     # all take the same time here
             assert r["candidates"] == len(gbscan.shape_candidates(b, kind))
+    """)
+
+
+def test_small_columns_are_cut_into_steps_of_their_decode(child):  # noqa: F811
+    child("""
+        def launched(n, b, layout, strategy):
+            c = gbscan.Column.from_packed(x, n, b, layout=layout)
+            c.run_async(0, 1, x, strategy)
+            return rt.fake_grid(), rt.fake_block_size() // 32
+
+        for strategy in ("branchfree", "branchy"):
+            for b, layout in ((8, "lanes"), (16, "lanes"), (20, "lanes"), (5, "rowmajor"), (16, "rowmajor"),
+                              (16, "bytes"), (20, "rowmajor")):
+                # blocks per step: four lanes a thread, two above 16 bits, one where a lane is a thread's
+                sliced = b <= (16 if strategy == "branchy" else 12 if layout == "lanes" else 8 if b in (8, 16) else 15)
+                step = 1 if sliced or (layout == "rowmajor" and b & (b - 1)) else 4 if b <= 16 else 2
+                for blocks in (1, 3, 4, 7):
+                    tiles = -(-blocks // step)
+                    assert launched(1024 * blocks, b, layout, strategy) == (1, tiles), (b, layout, strategy, blocks)
+                    if tiles < 8:                      # the tail takes a warp of its own
+                        assert launched(1024 * blocks + 5, b, layout, strategy) == (1, tiles + 1), (b, layout, strategy)
     """)
