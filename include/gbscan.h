@@ -415,7 +415,7 @@ uint64_t scan_planner_param_count(const scan_planner *planner);
  * resets the Adam state. */
 scan_status scan_planner_get_params(const scan_planner *planner, float *host_params);
 scan_status scan_planner_set_params(scan_planner *planner, const float *host_params);
-/* dev_y[rows x S] = network(dev_x[rows x 4]). */
+/* dev_y[rows x S] = network(dev_x[rows x 4]); the two may share memory. */
 scan_status scan_planner_forward(scan_planner *planner, const float *dev_x, uint32_t rows, float *dev_y,
                                  void *stream);
 /* Gradients of mean((y - t)^2) with respect to every parameter into dev_grads
